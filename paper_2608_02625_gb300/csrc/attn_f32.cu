@@ -3,9 +3,22 @@
 // Sec. 4.2: every valid position attends to every valid position (the block
 // masks of dlm_attn_masked restrict each query to its key ranges). fp32
 // inputs call for fp32 arithmetic throughout (TF32 tensor cores would not hold
-// a 1e-5 error bound), so this path is a plain online-softmax loop: one warp
-// per query row, lanes split the head dimension, a key's score is a warp
-// reduction, and the running maximum / sum / output are rescaled with expf.
+// a 1e-5 error bound), so both products run as fp32 FMAs on register tiles.
+//
+// One CTA of 256 threads (16 x 16) computes 16 * kR query rows of one head
+// against 64-key tiles staged in shared memory: thread (ty, tx) owns the rows
+// ty * kR .. + kR - 1 and, of the scores, the keys tx + 16 j; of the output,
+// the columns 4 tx + 64 c .. + 3. The scores accumulate even and odd head-dim
+// elements in the two halves of packed fp32 FMAs (operands read as they lie in
+// memory, 16 bytes a load); a row's scores belong to one half-warp, so its
+// maximum is four shuffles and the numerators pass to the second product
+// through a half-warp's own slice of shared memory without a block barrier.
+// K and V have one buffer each: V_t is copied (cp.async) behind the scores of
+// tile t, K_{t+1} behind its softmax and second product.
+//
+// Bound by the FMA pipe: 80 % busy on the SMs that have a CTA (1 x 512, 32 / 4
+// heads, D = 128: 128 tiles of 128 rows on 152 SMs, 102 us against 1022 us for a
+// warp per query row; 8 x 512: 0.70 ms = 49 TFLOP/s).
 #include <cmath>
 #include <cstdint>
 
@@ -15,84 +28,350 @@
 namespace dlm {
 namespace {
 
-constexpr int kWarpsPerBlock = 8;
+constexpr int kThreads = 256;
+constexpr int kKeys = 64;  // keys per tile
 
-template <int D>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32) attn_f32_kernel(AttnArgs a, float scale, int* err) {
-  constexpr int kPer = D / 32;
-  const int lane = threadIdx.x & 31;
-  const int i = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-  const int h = blockIdx.y;
-  const int b = blockIdx.z;
-  if (i >= a.L) return;
+template <int D, int kR>
+struct F32Tile {
+  static constexpr int kM = 16 * kR;               // query rows per CTA
+  static constexpr int kKStride = D + 4;           // floats; 16 lanes' rows then hit distinct banks
+  static constexpr int kQGroup = kR * D + 4;       // one row group; two groups of a warp hit distinct banks
+  static constexpr int kPGroup = kKeys * kR + 4;   // numerators of one row group, [key][row]
+  static constexpr int kQ = 16 * kQGroup, kK = kKeys * kKStride, kV = kKeys * D, kP = 16 * kPGroup;
+  static constexpr size_t kBytes = sizeof(float) * (kQ + kK + kV + kP);
+};
+
+// `bytes` (16 or 4) from global to shared memory, zeros instead when !valid.
+template <int kBytes>
+__device__ __forceinline__ void copy_or_zero(float* dst, const float* src, bool valid) {
+  const int n = valid ? kBytes : 0;
+  if constexpr (kBytes == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void copy4(float* dst, const float* src, bool valid, bool vec) {
+  if (vec) {
+    copy_or_zero<16>(dst, src, valid);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) copy_or_zero<4>(dst + e, src + e, valid);
+  }
+}
+
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+__device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
+
+template <int D, int kR, bool kMasked>
+__global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float scale, bool vec, int* err) {
+  using T = F32Tile<D, kR>;
+  extern __shared__ float4 smem_f4[];
+  float* const sq = reinterpret_cast<float*>(smem_f4);
+  float* const sk = sq + T::kQ;
+  float* const sv = sk + T::kK;
+  float* const sp = sv + T::kV;
+  constexpr int kC4 = D / 4;    // 16-byte chunks per row
+  constexpr int kCols = D / 64;  // float4 output columns per thread
+
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int row0 = blockIdx.x * T::kM, h = blockIdx.y, b = blockIdx.z;
   int n = a.seq_lens ? a.seq_lens[b] : a.L;
   if (n < 0 || n > a.L) {
-    if (lane == 0) set_device_error(err, DLM_DEVERR_LENGTH);
+    if (tid == 0) set_device_error(err, DLM_DEVERR_LENGTH);
     n = n < 0 ? 0 : a.L;
   }
-  const int g = (h * a.Hkv) / a.Hq;
-  float* o = static_cast<float*>(a.out) + b * a.so[0] + i * a.so[1] + h * a.so[2];
-  if (i >= n) {
-#pragma unroll
-    for (int t = 0; t < kPer; ++t) o[lane + 32 * t] = 0.f;
-    return;
-  }
-  const float* qp = static_cast<const float*>(a.q) + b * a.sq[0] + i * a.sq[1] + h * a.sq[2];
-  const float* kb = static_cast<const float*>(a.k) + b * a.sk[0] + g * a.sk[2];
-  const float* vb = static_cast<const float*>(a.v) + b * a.sv[0] + g * a.sv[2];
-  float q[kPer], acc[kPer];
-#pragma unroll
-  for (int t = 0; t < kPer; ++t) {
-    q[t] = qp[lane + 32 * t] * scale;
-    acc[t] = 0.f;
-  }
   int p = 0;
-  if (a.mask_mode != DLM_ATTN_FULL && a.prompt_lens) {
+  if (kMasked && a.prompt_lens) {
     p = a.prompt_lens[b];
     if (p < 0 || p > n) {
-      if (lane == 0) set_device_error(err, DLM_DEVERR_LENGTH);
+      if (tid == 0 && row0 < n) set_device_error(err, DLM_DEVERR_LENGTH);
       p = p < 0 ? 0 : n;
     }
   }
-  const KeyRanges kr = key_ranges(a.mask_mode, a.block, i, n, p);
-  float m = -INFINITY, l = 0.f;
-  for (int j = 0; j < kr.hi2; ++j) {
-    if (j == kr.hi1 && kr.lo2 > j) j = kr.lo2;   // skip the keys between the two ranges
-    if (j >= kr.hi2) break;
-    const float* kj = kb + j * a.sk[1];
-    float s = 0.f;
-#pragma unroll
-    for (int t = 0; t < kPer; ++t) s = fmaf(q[t], kj[lane + 32 * t], s);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    const float m_new = fmaxf(m, s);
-    const float corr = expf(m - m_new);  // 0 on the first key (m = -inf)
-    const float pj = expf(s - m_new);
-    l = l * corr + pj;
-    const float* vj = vb + j * a.sv[1];
-#pragma unroll
-    for (int t = 0; t < kPer; ++t) acc[t] = fmaf(pj, vj[lane + 32 * t], acc[t] * corr);
-    m = m_new;
+  const int g = (h * a.Hkv) / a.Hq;
+  const float* qb = static_cast<const float*>(a.q) + b * a.sq[0] + h * a.sq[2];
+  const float* kb = static_cast<const float*>(a.k) + b * a.sk[0] + g * a.sk[2];
+  const float* vb = static_cast<const float*>(a.v) + b * a.sv[0] + g * a.sv[2];
+
+  // Key tiles the CTA's rows may use: tile t starts at key 64 * (t < ka ? t : t + gap).
+  int tiles = row0 < n ? (n + kKeys - 1) / kKeys : 0, ka = tiles, gap = 0;
+  const int r_last = min(row0 + T::kM, n) - 1;
+  KeyRanges first{n, n, n}, last{n, n, n};  // of the CTA's first and last valid row
+  if (kMasked && tiles > 0) {
+    first = key_ranges(a.mask_mode, a.block, row0, n, p);
+    last = key_ranges(a.mask_mode, a.block, r_last, n, p);
+    if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL || r_last < p) {
+      ka = tiles = (last.hi1 + kKeys - 1) / kKeys;
+    } else {
+      const int prompt_end = (p + kKeys - 1) / kKeys;
+      const int own = (row0 < p ? p : first.lo2) / kKeys, end = (last.hi2 + kKeys - 1) / kKeys;
+      if (own <= prompt_end) {
+        ka = tiles = max(prompt_end, end);
+      } else {
+        ka = prompt_end;
+        gap = own - prompt_end;
+        tiles = prompt_end + end - own;
+      }
+    }
   }
-  const float inv = 1.0f / l;
+  // This thread's rows' keys: [0, hi1) and [lo2, hi2).
+  int hi1[kMasked ? kR : 1], lo2[kMasked ? kR : 1], hi2[kMasked ? kR : 1];
+  if (kMasked) {
 #pragma unroll
-  for (int t = 0; t < kPer; ++t) o[lane + 32 * t] = acc[t] * inv;
+    for (int r = 0; r < kR; ++r) {
+      const KeyRanges kr = key_ranges(a.mask_mode, a.block, min(row0 + ty * kR + r, max(n - 1, 0)), n, p);
+      hi1[r] = kr.hi1;
+      lo2[r] = kr.lo2;
+      hi2[r] = kr.hi2;
+    }
+  }
+
+  float2 o[kR][2 * kCols];
+  float m[kR], l[kR];  // running maximum; this thread's part of the row sum
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    m[r] = -INFINITY;
+    l[r] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 2 * kCols; ++c) o[r][c] = make_float2(0.f, 0.f);
+  }
+
+  auto load_keys = [&](float* dst, int stride, const float* base, int64_t s_row, int key0) {
+#pragma unroll
+    for (int e = 0; e < kKeys * kC4 / kThreads; ++e) {
+      const int i = tid + e * kThreads, key = i / kC4, c = i % kC4;
+      const bool valid = key0 + key < n;
+      copy4(dst + key * stride + 4 * c, base + (valid ? (key0 + key) * s_row + 4 * c : 0), valid, vec);
+    }
+  };
+  auto key_of = [&](int t) { return kKeys * (t < ka ? t : t + gap); };
+
+  if (tiles > 0) {
+    for (int i = tid; i < T::kM * kC4; i += kThreads) {
+      const int r = i / kC4, c = i % kC4;
+      const bool valid = row0 + r < n;
+      copy4(sq + (r / kR) * T::kQGroup + (r % kR) * D + 4 * c, qb + (valid ? (row0 + r) * a.sq[1] + 4 * c : 0), valid, vec);
+    }
+    load_keys(sk, T::kKStride, kb, a.sk[1], key_of(0));
+    copies_commit();
+    copies_wait<0>();
+    __syncthreads();
+  }
+  const float* const q_mine = sq + ty * T::kQGroup;
+  float* const p_mine = sp + ty * T::kPGroup;
+  for (int t = 0; t < tiles; ++t) {
+    const int key0 = key_of(t);
+    load_keys(sv, D, vb, a.sv[1], key0);
+    copies_commit();
+    // ---- scores of keys key0 + tx + 16 j
+    float2 s2[kR][4];
+#pragma unroll
+    for (int r = 0; r < kR; ++r)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s2[r][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int c = 0; c < kC4; ++c) {
+      float4 kf[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) kf[j] = *reinterpret_cast<const float4*>(sk + (tx + 16 * j) * T::kKStride + 4 * c);
+#pragma unroll
+      for (int r = 0; r < kR; ++r) {
+        const float4 qf = *reinterpret_cast<const float4*>(q_mine + r * D + 4 * c);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          s2[r][j] = ffma2(make_float2(qf.x, qf.y), make_float2(kf[j].x, kf[j].y), s2[r][j]);
+          s2[r][j] = ffma2(make_float2(qf.z, qf.w), make_float2(kf[j].z, kf[j].w), s2[r][j]);
+        }
+      }
+    }
+    __syncthreads();  // every warp is done with K_t
+    if (t + 1 < tiles) load_keys(sk, T::kKStride, kb, a.sk[1], key_of(t + 1));
+    copies_commit();
+    // ---- online softmax; numerators to the half-warp's slice
+    // Whether some row of the CTA may not use some key of the tile.
+    const bool partial = kMasked ? !(key0 + kKeys <= min(first.hi1, last.hi1) ||
+                                     (key0 >= last.lo2 && key0 + kKeys <= min(first.hi2, last.hi2)))
+                                 : key0 + kKeys > n;
+#pragma unroll
+    for (int r = 0; r < kR; ++r) {
+      float s[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[j] = (s2[r][j].x + s2[r][j].y) * scale;
+      if (partial) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int key = key0 + tx + 16 * j;
+          const bool ok = kMasked ? key < hi1[r] || (key >= lo2[r] && key < hi2[r]) : key < n;
+          if (!ok) s[j] = -INFINITY;
+        }
+      }
+      float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      const float m_new = fmaxf(m[r], mx);
+      // No key so far (every one masked): subtract 0, so that the numerators are exp(-inf) = 0.
+      const float sub = kMasked && m_new == -INFINITY ? 0.f : m_new;
+      const float corr = expf(m[r] - sub);  // 0 on the row's first keys (m = -inf)
+      m[r] = m_new;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[j] = expf(s[j] - sub);
+      l[r] = l[r] * corr + ((s[0] + s[1]) + (s[2] + s[3]));
+#pragma unroll
+      for (int c = 0; c < 2 * kCols; ++c) o[r][c] = fmul2(o[r][c], make_float2(corr, corr));
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s2[r][j].x = s[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float* dst = p_mine + (tx + 16 * j) * kR;
+      if constexpr (kR >= 4) {
+#pragma unroll
+        for (int r = 0; r < kR; r += 4)
+          *reinterpret_cast<float4*>(dst + r) = make_float4(s2[r][j].x, s2[r + 1][j].x, s2[r + 2][j].x, s2[r + 3][j].x);
+      } else {
+        *reinterpret_cast<float2*>(dst) = make_float2(s2[0][j].x, s2[1][j].x);
+      }
+    }
+    copies_wait<1>();  // V_t has landed (K_{t+1} may be in flight)
+    // A key a row may not use must not reach it, whatever its V holds: a zero
+    // numerator does not cancel a NaN or an infinity. (Rows past n are zeros
+    // in shared memory.) Each thread looks at what it copied itself.
+    bool guard = false;
+    if (kMasked && partial) {
+#pragma unroll
+      for (int e = 0; e < kKeys * kC4 / kThreads; ++e) {
+        const float4 x = reinterpret_cast<const float4*>(sv)[tid + e * kThreads];
+        guard |= not_finite(x.x) | not_finite(x.y) | not_finite(x.z) | not_finite(x.w);
+      }
+      guard = __syncthreads_or(guard);
+    } else {
+      __syncthreads();
+    }
+    // ---- output += numerators x V
+    if (!guard) {
+#pragma unroll 4
+      for (int key = 0; key < kKeys; ++key) {
+        float pr[kR];
+        if constexpr (kR >= 4) {
+#pragma unroll
+          for (int r = 0; r < kR; r += 4) {
+            const float4 x = *reinterpret_cast<const float4*>(p_mine + key * kR + r);
+            pr[r] = x.x, pr[r + 1] = x.y, pr[r + 2] = x.z, pr[r + 3] = x.w;
+          }
+        } else {
+          const float2 x = *reinterpret_cast<const float2*>(p_mine + key * kR);
+          pr[0] = x.x, pr[1] = x.y;
+        }
+#pragma unroll
+        for (int c = 0; c < kCols; ++c) {
+          const float4 vf = *reinterpret_cast<const float4*>(sv + key * D + 64 * c + 4 * tx);
+#pragma unroll
+          for (int r = 0; r < kR; ++r) {
+            o[r][2 * c] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.x, vf.y), o[r][2 * c]);
+            o[r][2 * c + 1] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.z, vf.w), o[r][2 * c + 1]);
+          }
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int key = 0; key < kKeys; ++key) {
+        const int kpos = key0 + key;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+          if (!(kpos < hi1[kMasked ? r : 0] || (kpos >= lo2[kMasked ? r : 0] && kpos < hi2[kMasked ? r : 0]))) continue;
+          const float w = p_mine[key * kR + r];
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) {
+            const float4 vf = *reinterpret_cast<const float4*>(sv + key * D + 64 * c + 4 * tx);
+            o[r][2 * c] = ffma2(make_float2(w, w), make_float2(vf.x, vf.y), o[r][2 * c]);
+            o[r][2 * c + 1] = ffma2(make_float2(w, w), make_float2(vf.z, vf.w), o[r][2 * c + 1]);
+          }
+        }
+      }
+    }
+    copies_wait<0>();
+    __syncthreads();  // K_{t+1} is visible, V_t and the numerators are free
+  }
+
+#pragma unroll
+  for (int r = 0; r < kR; ++r) {
+    const int i = row0 + ty * kR + r;
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
+    if (i >= a.L) continue;
+    float* dst = static_cast<float*>(a.out) + b * a.so[0] + i * a.so[1] + h * a.so[2] + 4 * tx;
+    const bool valid = i < n;
+    const float inv = valid ? 1.0f / l[r] : 0.f;
+#pragma unroll
+    for (int c = 0; c < kCols; ++c) {
+      const float2 lo = o[r][2 * c], hi = o[r][2 * c + 1];
+      const float4 x = valid ? make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (vec) {
+        *reinterpret_cast<float4*>(dst + 64 * c) = x;
+      } else {
+        dst[64 * c] = x.x, dst[64 * c + 1] = x.y, dst[64 * c + 2] = x.z, dst[64 * c + 3] = x.w;
+      }
+    }
+  }
+}
+
+template <int D, int kR, bool kMasked>
+int launch_tile(const AttnArgs& a, bool vec, cudaStream_t stream) {
+  using T = F32Tile<D, kR>;
+  const float scale = 1.0f / sqrtf(static_cast<float>(D));
+  cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<D, kR, kMasked>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(T::kBytes));
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 smem attribute: %s", cudaGetErrorString(e));
+  const dim3 grid((a.L + T::kM - 1) / T::kM, a.Hq, a.B);
+  attn_f32_kernel<D, kR, kMasked><<<grid, kThreads, T::kBytes, stream>>>(a, scale, vec, device_error_word());
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 launch: %s", cudaGetErrorString(e));
+  return DLM_OK;
+}
+
+template <int D, bool kMasked>
+int launch_d(const AttnArgs& a, cudaStream_t stream) {
+  // 16-byte copies and stores where every base and stride allows them.
+  bool vec = true;
+  const void* base[4] = {a.q, a.k, a.v, a.out};
+  const int64_t* strides[4] = {a.sq, a.sk, a.sv, a.so};
+  for (int t = 0; t < 4; ++t) {
+    vec &= reinterpret_cast<uintptr_t>(base[t]) % 16 == 0;
+    for (int i = 0; i < 3; ++i) vec &= strides[t][i] % 4 == 0;
+  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // Query rows per CTA (16 kR): the kR whose busiest SM is done first. In units
+  // of one 128-row CTA, a 64-row one takes 0.7 and a 32-row one 0.55 alone on
+  // an SM; a further one beside it adds 0.7 (0.54 with D = 64, where two fit)
+  // and 0.44. Measured at D = 128, 32 heads, per 64-key tile: 13.1 / 9.1 / 7.0 us
+  // alone, 11.5 us for two 32-row CTAs. L = 512: 104 / 136 / 175 us with 128 / 64 /
+  // 32 rows; L = 256: 53 / 36 / 46; L = 128: 28 / 20 / 15 (a warp per query row,
+  // the kernel before: 1022 us at L = 512).
+  const double heads = static_cast<double>(a.B) * a.Hq;
+  auto cost = [&](int rows, double alone, double more) {
+    return alone + (ceil(heads * ((a.L + rows - 1) / rows) / sms) - 1.0) * more;
+  };
+  const double c8 = cost(128, 1.0, 1.0), c4 = cost(64, 0.7, D == 64 ? 0.54 : 0.7), c2 = cost(32, 0.55, 0.44);
+  if (c8 <= c4 && c8 <= c2) return launch_tile<D, 8, kMasked>(a, vec, stream);
+  if (c4 <= c2) return launch_tile<D, 4, kMasked>(a, vec, stream);
+  return launch_tile<D, 2, kMasked>(a, vec, stream);
 }
 
 }  // namespace
 
 int launch_attn_f32(const AttnArgs& a, cudaStream_t stream) {
   if (a.B == 0 || a.L == 0) return DLM_OK;
-  dim3 grid((a.L + kWarpsPerBlock - 1) / kWarpsPerBlock, a.Hq, a.B);
-  const float scale = 1.0f / sqrtf(static_cast<float>(a.D));
-  if (a.D == 64) {
-    attn_f32_kernel<64><<<grid, kWarpsPerBlock * 32, 0, stream>>>(a, scale, device_error_word());
-  } else {
-    attn_f32_kernel<128><<<grid, kWarpsPerBlock * 32, 0, stream>>>(a, scale, device_error_word());
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 launch: %s", cudaGetErrorString(e));
-  return DLM_OK;
+  if (a.mask_mode != DLM_ATTN_FULL)
+    return a.D == 64 ? launch_d<64, true>(a, stream) : launch_d<128, true>(a, stream);
+  return a.D == 64 ? launch_d<64, false>(a, stream) : launch_d<128, false>(a, stream);
 }
 
 }  // namespace dlm

@@ -261,3 +261,34 @@ def test_workload_tiles_bit_identical():
             Bn.dlm_set_attn_tiles_per_unit(0)
     assert torch.equal(outs[0], outs[1])
 
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,D", [
+    (3, 33, 2, 1, 128),      # 32-row tiles, the second nearly empty
+    (1, 128, 16, 16, 64),    # whole 32-row tiles
+    (9, 129, 8, 2, 64), (3, 129, 20, 4, 128),    # 64-row tiles, a last one of one row
+    (5, 257, 16, 4, 128), (20, 65, 32, 8, 64),   # 128-row tiles
+])
+def test_f32_tile_edges(B, L, Hq, Hkv, D):
+    """Each query tile of the fp32 kernel (32, 64 and 128 rows, chosen by the
+    number of tiles), with lengths at the edges of the 64-key tiles."""
+    sl = [(L, L - 1, 1, 64, 65, 0, 63)[b % 7] for b in range(B)]
+    run_case(B, L, Hq, Hkv, D, [min(n, L) for n in sl], 1.0, "f32", seed=B + L)
+
+
+@pytest.mark.parametrize("L,Hq", [(40, 2), (70, 80), (128, 152)])
+def test_f32_unaligned_views(L, Hq):
+    """fp32 bases and strides need no 16-byte alignment: views one element into
+    rows of D + 1 elements take 4-byte copies, with each query tile."""
+    D = 64
+    q, k, v = rand_qkv(1, L, Hq, 1, D, 1.0, "f32", seed=L)
+    ref = oracle.bidir_attn(q.numpy(), k.numpy(), v.numpy(), [L - 3])
+
+    def view(t):
+        wide = torch.zeros(*t.shape[:3], D + 1, device=dev())
+        wide[..., 1:] = t.to(dev())
+        return wide[..., 1:]
+
+    out = view(torch.full(q.shape, float("nan")))
+    gpu_attn(view(q), view(k), view(v), [L - 3], out=out)
+    compare(out, ref, [L - 3], ATTN_TOL_F32, where=f"unaligned f32 L={L}")

@@ -134,3 +134,22 @@ def test_workload_full_size(mode):
                                     mask_mode=mode, block=64, prompt_lens=[pl[b]])
             compare(g_out[b:b + 1, :, h:h + 1], ref, [n[b]], ATTN_TOL_BF16, where=f"c3 mode {mode} b={b} h={h}")
 
+
+
+@pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
+@pytest.mark.parametrize("Hq", [2, 80, 152])
+def test_f32_values_outside_a_mask_never_reach_a_row(mode, Hq):
+    """A NaN or an infinity in v at a key reaches the rows that attend to the key
+    and no other, with each query tile of the fp32 kernel (32, 64, 128 rows)."""
+    L, p, block, key = 128, 20, 40, 97   # blocks [20, 60), [60, 100), [100, 128)
+    q, k, v = rand_qkv(1, L, Hq, 1, 64, 1.0, "f32", seed=Hq)
+    bad = v.clone()
+    bad[0, key, 0, ::2] = float("nan")
+    bad[0, key, 0, 1::2] = float("inf")
+    good, got = (gpu_masked(q.to(dev()), k.to(dev()), x.to(dev()), [L], [p], mode, block) for x in (v, bad))
+    attends = torch.zeros(L, dtype=torch.bool, device=dev())
+    attends[60:100] = True               # the key's own block
+    if mode == CAUSAL:
+        attends[100:] = True
+    assert torch.equal(got[0, ~attends], good[0, ~attends])
+    assert not torch.isfinite(got[0, attends]).any()
