@@ -139,6 +139,40 @@ int* device_error_word() {
   return g_err_addr[dev];
 }
 
+int active_clusters(const void* kernel, int csize, int threads, size_t smem) {
+  struct Known {
+    const void* kernel;
+    int dev, csize, clusters;
+  };
+  constexpr int kMax = 256;
+  static std::mutex mu;
+  static Known known[kMax];
+  static int count = 0;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  for (int i = 0; i < count; ++i)
+    if (known[i].kernel == kernel && known[i].dev == dev && known[i].csize == csize) return known[i].clusters;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(csize * sms));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if ((csize > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  if (count < kMax) known[count++] = {kernel, dev, csize, n};
+  return n;
+}
+
 }  // namespace dlm
 
 namespace {

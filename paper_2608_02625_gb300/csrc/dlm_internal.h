@@ -31,6 +31,11 @@ void clear_error();
 // The calling thread's stream (dlm_set_stream).
 cudaStream_t current_stream();
 
+// Clusters of `csize` CTAs of `kernel` (`threads` each, `smem` bytes of dynamic
+// shared memory, `csize` up to 16) that run at once on the current device, 0
+// if none can; asked of the runtime once per device, kernel and size.
+int active_clusters(const void* kernel, int csize, int threads, size_t smem);
+
 struct AttnArgs {
   const void* q;
   const void* k;
@@ -104,9 +109,8 @@ struct LmArgs {
   void* workspace;      // lmhead_workspace_bytes(N)
 };
 
-constexpr int kLmMaxSplits = 64;
+constexpr int kLmMaxSplits = 64;  // parts per row in the workspace
 inline size_t lmhead_workspace_bytes(int64_t N) { return static_cast<size_t>(N) * kLmMaxSplits * 12; }
-int lmhead_splits(int64_t N, int64_t V, int sms);
 int launch_lmhead(const LmArgs& a, cudaStream_t stream);
 
 }  // namespace dlm

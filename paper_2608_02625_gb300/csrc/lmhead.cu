@@ -23,9 +23,15 @@
 //              running sum of exp(x - m) when the maximum grows, and adds the
 //              chunk's terms (per-tile partial sums keep the fp32 sum short)
 // At the end of an item each row's (max, first index, sum) is written to the
-// caller's workspace; lmhead_combine_kernel merges the splits of a row in
-// vocabulary order (ties keep the lower index). Every mbarrier wait is
+// caller's workspace; lmhead_combine_kernel merges the parts of a row (ties
+// keep the lower index). The workspace has kLmMaxSplits parts per row, fewer
+// than there are SMs: with one or two row blocks (a local window, a single
+// position: bound by reading the weight) the vocabulary is split over clusters
+// of CTAs, which merge their rows' parts through distributed shared memory
+// before one part is written, so that every SM reads a share of the weight.
+// Every mbarrier wait is
 // bounded; on expiry the kernel sets DLM_DEVERR_TIMEOUT, drains and exits.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -35,6 +41,8 @@
 
 #include "dlm_common.cuh"
 #include "dlm_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace dlm {
 namespace {
@@ -46,7 +54,7 @@ constexpr int kStages = 4;
 constexpr int kThreads = 256;     // warp 0 TMA, warp 1 MMA, warps 4-7 epilogue
 constexpr int kEpiWarp0 = 4;
 constexpr uint32_t kTmemCols = 512;
-constexpr int kABytes = kBM * kBK * 2;  // 16 KB
+constexpr int kABytes = kBM * kBK * 2;  // 16 KB (a stage of it holds LmParams::a_rows rows)
 constexpr int kBBytes = kBN * kBK * 2;  // 32 KB
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -58,13 +66,18 @@ struct Smem {
   uint64_t acc_full[2];       // accumulator complete     (MMA -> epilogue)
   uint64_t acc_empty[2];      // accumulator read out     (epilogue -> MMA)
   uint64_t done;              // every MMA completed      (teardown)
+  float part_m[kBM], part_s[kBM];  // this CTA's part of each row, read by rank 0 of its cluster
+  int part_idx[kBM];
   uint32_t tmem_base;
   int abort;
 };
 
 struct LmParams {
   int N, V, d;
-  int row_blocks, vtiles, splits, items;
+  int row_blocks, vtiles, items;
+  int csize;    // CTAs per cluster; above 1 a cluster runs one item
+  int splits;   // vocabulary splits: csize per part written
+  int a_rows;   // rows of the hidden box: 128, or N rounded up to 8 when smaller
   float* part_m;
   int* part_idx;
   float* part_s;
@@ -73,16 +86,31 @@ struct LmParams {
 };
 
 struct Item {
-  int rb, split, t0, t1;  // row block, split, vocabulary tiles [t0, t1)
+  int rb, part, t0, t1;  // row block, part written, vocabulary tiles [t0, t1)
 };
 
-__device__ __forceinline__ Item item_at(const LmParams& p, int item) {
+// Share of cluster rank `rank` of work item `item` (a part and a row block).
+__device__ __forceinline__ Item item_at(const LmParams& p, int item, int rank) {
   Item it;
-  it.split = item / p.row_blocks;
+  it.part = item / p.row_blocks;
   it.rb = item % p.row_blocks;
-  it.t0 = static_cast<int>(static_cast<long long>(p.vtiles) * it.split / p.splits);
-  it.t1 = static_cast<int>(static_cast<long long>(p.vtiles) * (it.split + 1) / p.splits);
+  const int split = it.part * p.csize + rank;
+  it.t0 = static_cast<int>(static_cast<long long>(p.vtiles) * split / p.splits);
+  it.t1 = static_cast<int>(static_cast<long long>(p.vtiles) * (split + 1) / p.splits);
   return it;
+}
+
+// Merges another part (m2, idx2, s2) of a row into (m, idx, s); the lower
+// vocabulary index wins equal maxima.
+__device__ __forceinline__ void merge_part(float& m, int& idx, float& s, float m2, int idx2, float s2) {
+  if (m2 > m) {
+    s = (m == -INFINITY ? 0.f : s * expf(m - m2)) + s2;
+    m = m2;
+    idx = idx2;
+  } else if (m2 != -INFINITY) {
+    s += s2 * expf(m2 - m);
+    if (m2 == m) idx = min(idx, idx2);
+  }
 }
 
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int* err,
@@ -98,6 +126,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int kblocks = p.d / kBK;
+  const int rank = static_cast<int>(blockIdx.x) % p.csize;
+  const int walker = static_cast<int>(blockIdx.x) / p.csize, walkers = static_cast<int>(gridDim.x) / p.csize;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -131,8 +161,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     int fill = 0;
     bool ok = true;
-    for (int item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-      const Item it = item_at(p, item);
+    for (int item = walker; ok && item < p.items; item += walkers) {
+      const Item it = item_at(p, item, rank);
       for (int vt = it.t0; ok && vt < it.t1; ++vt) {
         for (int kb = 0; kb < kblocks; ++kb, ++fill) {
           const int st = fill % kStages;
@@ -141,7 +171,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           if (lane == 0) {
-            mbar_arrive_expect_tx(&sm.full[st], kABytes + kBBytes);
+            mbar_arrive_expect_tx(&sm.full[st], p.a_rows * (kBK * 2) + kBBytes);
             tma_load_2d(sm.a[st], &th, &sm.full[st], kb * kBK, it.rb * kBM);
             tma_load_2d(sm.b[st], &tw, &sm.full[st], kb * kBK, vt * kBN);
           }
@@ -164,8 +194,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       constexpr uint32_t idesc = idesc_bf16_f32(kBM, kBN, false, false);  // both operands K-major
       int fill = 0, tile = 0;
       bool ok = true;
-      for (int item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-        const Item it = item_at(p, item);
+      for (int item = walker; ok && item < p.items; item += walkers) {
+        const Item it = item_at(p, item, rank);
         for (int vt = it.t0; ok && vt < it.t1; ++vt, ++tile) {
           const int acc = tile & 1;
           // The accumulator's previous tile (tile - 2) must have been read out.
@@ -205,10 +235,12 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_base = static_cast<uint32_t>(qw * 32) << 16;
     int tile = 0;
     bool ok = true;
-    for (int item = blockIdx.x; ok && item < p.items; item += gridDim.x) {
-      const Item it = item_at(p, item);
+    for (int item = walker; ok && item < p.items; item += walkers) {
+      const Item it = item_at(p, item, rank);
       float m = -INFINITY, s = 0.f;
       int idx = 0;
+      const int row = it.rb * kBM + t;
+      const bool rows = row - lane < p.N;  // some row of this warp exists
       for (int vt = it.t0; vt < it.t1; ++vt, ++tile) {
         const int acc = tile & 1;
         if (!warp_wait(&sm.acc_full[acc], (tile >> 1) & 1, abort, p.err, p.wait_ns)) {
@@ -216,6 +248,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc_fence_after();
+        if (!rows) {
+          tc_fence_before();
+          mbar_arrive(&sm.acc_empty[acc]);
+          continue;
+        }
         const uint32_t base = tmem + lane_base + acc * kBN;
         float ts = 0.f;  // this tile's terms, relative to m
 #pragma unroll 1
@@ -260,9 +297,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         s += ts;
       }
       if (!ok) break;
-      const int row = it.rb * kBM + t;
-      if (row < p.N) {
-        const int64_t o = static_cast<int64_t>(it.split) * p.N + row;
+      if (p.csize > 1) {
+        sm.part_m[t] = m;
+        sm.part_idx[t] = idx;
+        sm.part_s[t] = s;
+      } else if (row < p.N) {
+        const int64_t o = static_cast<int64_t>(it.part) * p.N + row;
         p.part_m[o] = m;
         p.part_idx[o] = idx;
         p.part_s[o] = s;
@@ -270,6 +310,28 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
 
+  if (p.csize > 1) {
+    // Rank 0 merges the cluster's parts of each row; the second barrier keeps
+    // the other CTAs' shared memory alive until it has read them.
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (rank == 0 && warp >= kEpiWarp0) {
+      const Item it = item_at(p, walker, 0);
+      const int t = threadIdx.x - kEpiWarp0 * 32, row = it.rb * kBM + t;
+      if (row < p.N) {
+        float m = sm.part_m[t], s = sm.part_s[t];
+        int idx = sm.part_idx[t];
+        for (int r = 1; r < p.csize; ++r)
+          merge_part(m, idx, s, *cluster.map_shared_rank(&sm.part_m[t], r), *cluster.map_shared_rank(&sm.part_idx[t], r),
+                     *cluster.map_shared_rank(&sm.part_s[t], r));
+        const int64_t o = static_cast<int64_t>(it.part) * p.N + row;
+        p.part_m[o] = m;
+        p.part_idx[o] = idx;
+        p.part_s[o] = s;
+      }
+    }
+    cluster.sync();
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -278,28 +340,42 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// Merges the splits of each row in vocabulary order.
-__global__ void lmhead_combine_kernel(const float* part_m, const int* part_idx, const float* part_s, int N,
-                                      int splits, int32_t* argmax, float* conf, float* lse) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+// Merges the parts of each row, one warp per row: the parts' loads are all in
+// flight at once. (One thread per row walking its 64 parts took ~40 us, the
+// latency of a chain of loads, where the projection of 64 rows takes ~95.)
+constexpr int kCombineThreads = 256;
+__global__ void __launch_bounds__(kCombineThreads)
+    lmhead_combine_kernel(const float* part_m, const int* part_idx, const float* part_s, int N, int parts,
+                          int32_t* argmax, float* conf, float* lse) {
+  const int64_t r = (static_cast<int64_t>(blockIdx.x) * kCombineThreads + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (r >= N) return;
-  float m = -INFINITY, s = 0.f;
-  int idx = 0;
-  for (int k = 0; k < splits; ++k) {
+  constexpr int kPer = kLmMaxSplits / 32;
+  float pm[kPer], ps[kPer];
+  int pi[kPer];
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const int k = lane + 32 * j;
     const int64_t o = static_cast<int64_t>(k) * N + r;
-    const float mk = part_m[o];
-    const float sk = part_s[o];
-    if (mk > m) {
-      s = (m == -INFINITY ? 0.f : s * expf(m - mk)) + sk;
-      m = mk;
-      idx = part_idx[o];
-    } else if (mk != -INFINITY) {
-      s += sk * expf(mk - m);
-    }
+    pm[j] = k < parts ? part_m[o] : -INFINITY;
+    pi[j] = k < parts ? part_idx[o] : 0x7FFFFFFF;
+    ps[j] = k < parts ? part_s[o] : 0.f;
   }
-  argmax[r] = idx;
-  conf[r] = 1.0f / s;
-  lse[r] = m + logf(s);
+  float m = pm[0], s = ps[0];
+  int idx = pi[0];
+#pragma unroll
+  for (int j = 1; j < kPer; ++j) merge_part(m, idx, s, pm[j], pi[j], ps[j]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
+    const int idx2 = __shfl_xor_sync(0xffffffffu, idx, o);
+    merge_part(m, idx, s, m2, idx2, s2);
+  }
+  if (lane == 0) {
+    argmax[r] = idx;
+    conf[r] = 1.0f / s;
+    lse[r] = m + logf(s);
+  }
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -337,23 +413,40 @@ int make_map_2d(CUtensorMap* map, const void* base, int64_t rows, int d, int64_t
 
 }  // namespace
 
-int lmhead_splits(int64_t N, int64_t V, int sms) {
-  const int64_t row_blocks = (N + kBM - 1) / kBM;
-  const int64_t vtiles = (V + kBN - 1) / kBN;
-  int best = 1;
+namespace {
+
+struct Split {
+  int csize, parts;  // CTAs per cluster, parts per row
+};
+
+// The split that leaves the busiest CTA the fewest 256-column tiles, plus a
+// small cost per item (pipeline fill, flush). Clusters (csize > 1) run one
+// item each, all at once. Measured for 64 rows x 151552 x 2048 (reading the
+// weight at the HBM copy rate: 93 us): 64 single CTAs 127 us, 64 clusters of 2
+// 101 us, 50 of 3 101 us, 32 of 4 101 us; 37 of 4, which are not all resident at
+// once, 141 us. 200 rows: 154 us with single CTAs, 117 us. From three row
+// blocks on, single CTAs fill the SMs.
+Split choose_split(int64_t row_blocks, int64_t vtiles, int sms, size_t smem) {
+  Split best{1, 1};
   double best_cost = 1e300;
-  for (int s = 1; s <= kLmMaxSplits && s <= vtiles; ++s) {
-    const int64_t items = row_blocks * s;
-    const int64_t rounds = (items + sms - 1) / sms;
-    // Tiles on the busiest CTA, plus a small cost per item (pipeline fill, flush).
-    const double cost = static_cast<double>(rounds) * (static_cast<double>((vtiles + s - 1) / s) + 0.5);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = s;
+  for (int c = 1; c <= 4; c *= 2) {
+    if (c > 1 && row_blocks * kLmMaxSplits >= sms) break;  // single CTAs already fill the SMs
+    const int64_t active = c == 1 ? sms : active_clusters(reinterpret_cast<const void*>(lmhead_kernel), c, kThreads, smem);
+    for (int s = 1; s <= kLmMaxSplits && s <= (vtiles + c - 1) / c; ++s) {  // a cluster's last CTAs may have no tile
+      const int64_t items = row_blocks * s;
+      if (c > 1 && items > active) break;
+      const int64_t rounds = (items + active - 1) / active;
+      const double cost = static_cast<double>(rounds) * (static_cast<double>((vtiles + s * c - 1) / (s * c)) + 0.5);
+      if (cost < best_cost - 1e-9) {
+        best_cost = cost;
+        best = {c, s};
+      }
     }
   }
   return best;
 }
+
+}  // namespace
 
 int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
   if (a.N == 0) return DLM_OK;
@@ -366,28 +459,40 @@ int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
   p.d = static_cast<int>(a.d);
   p.row_blocks = static_cast<int>((a.N + kBM - 1) / kBM);
   p.vtiles = static_cast<int>((a.V + kBN - 1) / kBN);
-  p.splits = lmhead_splits(a.N, a.V, sms);
-  p.items = p.row_blocks * p.splits;
-  float* ws = static_cast<float*>(a.workspace);
-  p.part_m = ws;
-  p.part_idx = reinterpret_cast<int*>(ws + static_cast<int64_t>(p.splits) * a.N);
-  p.part_s = ws + 2 * static_cast<int64_t>(p.splits) * a.N;
-  p.err = device_error_word();
-  p.wait_ns = wait_budget_ns();
-  CUtensorMap mh, mw;
-  int st;
-  if ((st = make_map_2d(&mh, a.hidden, a.N, p.d, a.s_hidden, kBM)) != DLM_OK) return st;
-  if ((st = make_map_2d(&mw, a.weight, a.V, p.d, a.s_weight, kBN)) != DLM_OK) return st;
+  p.a_rows = a.N < kBM ? static_cast<int>((a.N + 7) / 8 * 8) : kBM;
   const size_t smem = sizeof(Smem) + 1024;
   cudaError_t e = cudaFuncSetAttribute(lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead smem attribute: %s", cudaGetErrorString(e));
-  const int grid = p.items < sms ? p.items : sms;
-  lmhead_kernel<<<grid, kThreads, smem, stream>>>(mh, mw, p);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead launch: %s", cudaGetErrorString(e));
-  lmhead_combine_kernel<<<static_cast<unsigned>((a.N + 255) / 256), 256, 0, stream>>>(
-      p.part_m, p.part_idx, p.part_s, p.N, p.splits, a.argmax, a.conf, a.lse);
+  Split sp = choose_split(p.row_blocks, p.vtiles, sms, smem);
+  p.csize = sp.csize;
+  p.splits = sp.parts * sp.csize;
+  p.items = p.row_blocks * sp.parts;
+  float* ws = static_cast<float*>(a.workspace);
+  p.part_m = ws;
+  p.part_idx = reinterpret_cast<int*>(ws + static_cast<int64_t>(sp.parts) * a.N);
+  p.part_s = ws + 2 * static_cast<int64_t>(sp.parts) * a.N;
+  p.err = device_error_word();
+  p.wait_ns = wait_budget_ns();
+  CUtensorMap mh, mw;
+  int st;
+  if ((st = make_map_2d(&mh, a.hidden, a.N, p.d, a.s_hidden, p.a_rows)) != DLM_OK) return st;
+  if ((st = make_map_2d(&mw, a.weight, a.V, p.d, a.s_weight, kBN)) != DLM_OK) return st;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(sp.csize > 1 ? p.items * sp.csize : (p.items < sms ? p.items : sms)));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {static_cast<unsigned>(sp.csize), 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = sp.csize > 1 ? 1 : 0;
+  if ((e = cudaLaunchKernelEx(&cfg, lmhead_kernel, mh, mw, p)) != cudaSuccess)
+    return fail(DLM_ERR_CUDA, "lmhead launch: %s", cudaGetErrorString(e));
+  const unsigned combine_grid = static_cast<unsigned>((a.N * 32 + kCombineThreads - 1) / kCombineThreads);
+  lmhead_combine_kernel<<<combine_grid, kCombineThreads, 0, stream>>>(p.part_m, p.part_idx, p.part_s, p.N, sp.parts,
+                                                                      a.argmax, a.conf, a.lse);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead combine launch: %s", cudaGetErrorString(e));
   return DLM_OK;

@@ -122,3 +122,20 @@ def test_full_size_sampled_rows():
     rng = np.random.default_rng(3)
     rows = np.unique(np.concatenate([[0, 127, 128, N - 1], rng.integers(0, N, 20)]))
     check(tuple(a[rows] for a in gpu), hb[rows].float().numpy(), wb.float().numpy(), "full size")
+
+
+@pytest.mark.parametrize("N", [1, 8, 9, 64, 127, 128, 129, 256])
+@pytest.mark.parametrize("V", [257, 16384 + 1, 33000])
+def test_few_row_blocks_split_over_clusters(N, V):
+    """One and two row blocks: a hidden box of N rounded up to 8 rows, the
+    vocabulary split over clusters of CTAs (the last of which may have no tile),
+    whose parts meet in one CTA. Duplicate weight rows put exactly equal maxima
+    in different CTAs of a cluster and in different clusters."""
+    hb, wb = make_inputs(N, V, 64, seed=N + V, peak_frac=0.5, peak=10.0)
+    am = oracle.lm_head_confidence(hb.float().numpy(), wb.float().numpy())[0].astype(np.int64)
+    wb[torch.from_numpy((am + 256) % V)] = wb[torch.from_numpy(am)]       # the next tile
+    wb[torch.from_numpy((am + V // 2) % V)] = wb[torch.from_numpy(am)]    # another cluster
+    gpu = gpu_lmhead(hb.to(dev()), wb.to(dev()))
+    check(gpu, hb.float().numpy(), wb.float().numpy(), f"N={N} V={V}")
+    ref_am = oracle.lm_head_confidence(hb.float().numpy(), wb.float().numpy())[0]
+    np.testing.assert_array_equal(gpu[0], ref_am)
