@@ -4,8 +4,12 @@ Each function has the name and argument order of its C entry point
 (include/dlmrefine.h), takes torch CUDA tensors, builds the dlm_tensor
 descriptors, sets the library's stream to torch's current stream of the
 tensors' device and calls the library. All computation runs in the CUDA
-kernels; a nonzero status raises DlmError. The shared library must have been
+kernels; a nonzero status raises DlmError. The shared libraries must have been
 built (``python -m paper_2608_02625_gb300.build``): there is no fallback.
+
+The compute calls marshal natively (csrc/marshal.cpp) where their arguments are
+plain CUDA tensors on the current device; a call with any other argument goes
+through ctypes below, which accepts and refuses the same forms.
 """
 from __future__ import annotations
 
@@ -84,6 +88,7 @@ def _load():
 
 
 lib = _load()
+from . import _marshal  # noqa: E402  (native marshalling; links against the library loaded above)
 
 
 def describe(t: torch.Tensor | None) -> DlmTensor | None:
@@ -112,6 +117,14 @@ def _check(status: int):
     if status != 0:
         msg = lib.dlm_last_error().decode() or lib.dlm_status_string(status).decode()
         raise DlmError(status, msg)
+
+
+def _done(status) -> bool:
+    """Whether the native marshalling took a call (None: it did nothing)."""
+    if status is None:
+        return False
+    _check(status)
+    return True
 
 
 def _prepare(*tensors):
@@ -143,6 +156,8 @@ def dlm_status_string(status: int) -> str:
 
 def dlm_bidir_attn(q, k, v, seq_lens, out):
     """Non-causal GQA attention: out[b,i,h] = softmax(q k^T / sqrt(D)) v over keys j < n_b."""
+    if _done(_marshal.bidir_attn(q, k, v, seq_lens, out)):
+        return out
     _prepare(q, k, v, seq_lens, out)
     dq, dk, dv, ds, do = (describe(t) for t in (q, k, v, seq_lens, out))
     _check(lib.dlm_bidir_attn(_ref(dq), _ref(dk), _ref(dv), _ref(ds), _ref(do)))
@@ -155,6 +170,8 @@ ATTN_FULL, ATTN_BLOCK_CAUSAL, ATTN_BLOCK_LOCAL = 0, 1, 2
 def dlm_attn_masked(q, k, v, seq_lens, prompt_lens, mode: int, block: int, out):
     """Attention restricted by a block mask (ATTN_BLOCK_CAUSAL: prompt, earlier
     blocks and the own block; ATTN_BLOCK_LOCAL: prompt and the own block)."""
+    if _done(_marshal.attn_masked(q, k, v, seq_lens, prompt_lens, mode, block, out)):
+        return out
     _prepare(q, k, v, seq_lens, prompt_lens, out)
     ds = [describe(t) for t in (q, k, v, seq_lens, prompt_lens)]
     do = describe(out)
@@ -164,6 +181,8 @@ def dlm_attn_masked(q, k, v, seq_lens, prompt_lens, mode: int, block: int, out):
 
 def dlm_vocab_confidence(logits, argmax, conf, lse):
     """Per row: argmax (lowest index), max softmax probability, log-sum-exp."""
+    if _done(_marshal.vocab_confidence(logits, argmax, conf, lse)):
+        return argmax, conf, lse
     _prepare(logits, argmax, conf, lse)
     ds = [describe(t) for t in (logits, argmax, conf, lse)]
     _check(lib.dlm_vocab_confidence(*[_ref(d) for d in ds]))
@@ -187,8 +206,13 @@ class RefineParams:
                                int(self.mask_id), self.prompt_lens.data_ptr(), self.seq_lens.data_ptr())
 
 
+_marshal.set_params_type(RefineParams)
+
+
 def dlm_refine_update(tokens, mask, argmax, conf, params: RefineParams, new_tokens, new_mask, n_edits):
     """Commit masked positions, edit confident changes, remask the k least confident."""
+    if _done(_marshal.refine_update(tokens, mask, argmax, conf, params, new_tokens, new_mask, n_edits)):
+        return new_tokens, new_mask, n_edits
     _prepare(tokens, mask, argmax, conf, new_tokens, new_mask, n_edits, params.prompt_lens, params.seq_lens)
     ds = [describe(t) for t in (tokens, mask, argmax, conf)]
     outs = [describe(t) for t in (new_tokens, new_mask, n_edits)]
@@ -203,6 +227,8 @@ def dlm_lmhead_workspace_bytes(rows: int) -> int:
 
 def dlm_lmhead_confidence(hidden, weight, argmax, conf, lse, workspace):
     """argmax / conf / lse of hidden @ weight^T per row, without materialising the logits."""
+    if _done(_marshal.lmhead_confidence(hidden, weight, argmax, conf, lse, workspace)):
+        return argmax, conf, lse
     _prepare(hidden, weight, argmax, conf, lse, workspace)
     if not workspace.is_contiguous():
         raise ValueError("workspace must be contiguous")
@@ -215,6 +241,8 @@ def dlm_lmhead_confidence(hidden, weight, argmax, conf, lse, workspace):
 
 def dlm_token_prob(logits, tokens, lse, prob):
     """prob[r] = exp(logits[r, tokens[r]] - lse[r]) (0 for a token outside [0, V))."""
+    if _done(_marshal.token_prob(logits, tokens, lse, prob)):
+        return prob
     _prepare(logits, tokens, lse, prob)
     ds = [describe(t) for t in (logits, tokens, lse, prob)]
     _check(lib.dlm_token_prob(*[_ref(d) for d in ds]))
@@ -224,6 +252,9 @@ def dlm_token_prob(logits, tokens, lse, prob):
 def dlm_refine_update_ranked(tokens, mask, argmax, conf, tok_prob, params: RefineParams, new_tokens, new_mask,
                              n_edits):
     """dlm_refine_update remasking by the probability of each position's resulting token."""
+    if _done(_marshal.refine_update_ranked(tokens, mask, argmax, conf, tok_prob, params, new_tokens,
+                                           new_mask, n_edits)):
+        return new_tokens, new_mask, n_edits
     _prepare(tokens, mask, argmax, conf, tok_prob, new_tokens, new_mask, n_edits, params.prompt_lens,
              params.seq_lens)
     ds = [describe(t) for t in (tokens, mask, argmax, conf, tok_prob)]
@@ -243,6 +274,9 @@ def dlm_refine_step(logits, tokens, mask, params: RefineParams, argmax, conf, ls
 
     workspace: a CUDA tensor of at least dlm_refine_step_workspace_bytes(B) bytes,
     zero before its first use; each completed call leaves it zero again."""
+    if _done(_marshal.refine_step(logits, tokens, mask, params, argmax, conf, lse, new_tokens, new_mask,
+                                  n_edits, workspace)):
+        return argmax, conf, lse, new_tokens, new_mask, n_edits
     _prepare(logits, tokens, mask, argmax, conf, lse, new_tokens, new_mask, n_edits, workspace,
              params.prompt_lens, params.seq_lens)
     if not workspace.is_contiguous():
@@ -262,6 +296,9 @@ def dlm_refine_step_static(logits, tokens, mask, params: RefineParams, argmax, c
     for callers that cannot allocate device memory. The first call on a device
     sets that device up (make it before any stream capture); calls that overlap
     on the GPU race on the shared scratch."""
+    if _done(_marshal.refine_step_static(logits, tokens, mask, params, argmax, conf, lse, new_tokens,
+                                         new_mask, n_edits)):
+        return argmax, conf, lse, new_tokens, new_mask, n_edits
     _prepare(logits, tokens, mask, argmax, conf, lse, new_tokens, new_mask, n_edits, params.prompt_lens,
              params.seq_lens)
     ins = [describe(t) for t in (logits, tokens, mask)]
@@ -285,6 +322,8 @@ class RefineLoop:
         holds the number of passes once the stream reaches that point."""
         if not self._h:
             raise ValueError("the loop has been destroyed")
+        if _done(_marshal.loop_launch(self._h, self.device.index)):
+            return
         torch.cuda.set_device(self.device)
         _check(lib.dlm_set_stream(ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)))
         _check(lib.dlm_loop_launch(ctypes.c_void_p(self._h)))

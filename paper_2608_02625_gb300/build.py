@@ -1,4 +1,5 @@
-"""Builds libdlmrefine.so and libdlmsynth.so in-tree for sm_103a (GB300).
+"""Builds libdlmrefine.so, libdlmsynth.so and the binding's native marshalling
+(_marshal.so) in-tree for sm_103a (GB300).
 
     python -m paper_2608_02625_gb300.build [--force] [--verbose] [--check-bounds --out DIR]
 
@@ -34,6 +35,8 @@ LIBS = {
                         "selftest.cu"],
     "libdlmsynth.so": ["synth.cu"],
 }
+# The Python binding's marshalling: host code against torch's headers, beside the library it calls.
+MARSHAL, MARSHAL_SRC = "_marshal.so", "marshal.cpp"
 HEADERS = ["dlm_common.cuh", "dlm_internal.h", "update_impl.cuh"]
 
 
@@ -69,6 +72,40 @@ def _compile(src: str, verbose: bool, check_bounds: bool = False) -> tuple[str, 
     return obj, r.stdout + r.stderr
 
 
+def _marshal_stale(force: bool) -> bool:
+    src, out = os.path.join(CSRC, MARSHAL_SRC), os.path.join(PKG, MARSHAL)
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(INCLUDE, "dlmrefine.h")))
+    return force or not os.path.exists(out) or os.path.getmtime(out) < newest
+
+
+def _host_cxx(args: list[str]) -> None:
+    r = subprocess.run([os.environ.get("CXX", "g++")] + args, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"{MARSHAL_SRC} failed to build:\n{r.stdout}\n{r.stderr}")
+
+
+def _compile_marshal() -> str:
+    import sysconfig
+
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    obj = os.path.join(BUILD, MARSHAL_SRC.replace(".cpp", ".o"))
+    dirs = [INCLUDE, inc, os.path.join(inc, "torch", "csrc", "api", "include"),
+            os.path.join(os.path.dirname(os.path.dirname(nvcc())), "include"), sysconfig.get_paths()["include"]]
+    _host_cxx(["-O2", "-fPIC", "-std=c++17", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"] +
+              [f"-I{d}" for d in dirs] + ["-c", os.path.join(CSRC, MARSHAL_SRC), "-o", obj])
+    return obj
+
+
+def _link_marshal(obj: str) -> None:
+    import torch
+    tlib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    out = os.path.join(PKG, MARSHAL)
+    _host_cxx(["-shared", obj, "-o", out + ".tmp", "-L" + PKG, "-ldlmrefine", "-Wl,-rpath,$ORIGIN", "-L" + tlib,
+               "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + tlib])
+    os.replace(out + ".tmp", out)
+
+
 def build(force: bool = False, verbose: bool = False, check_bounds: bool = False, out_dir: str | None = None) -> dict:
     out_dir = out_dir or PKG
     if check_bounds and os.path.abspath(out_dir) == PKG:
@@ -81,10 +118,12 @@ def build(force: bool = False, verbose: bool = False, check_bounds: bool = False
         if force or not os.path.exists(out) or os.path.getmtime(out) < _newest_input(srcs):
             todo[lib] = srcs
     logs = {}
-    if not todo:
+    marshal = out_dir == PKG and not check_bounds and _marshal_stale(force)
+    if not todo and not marshal:
         return logs
     srcs = sorted({s for v in todo.values() for s in v})
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=8) as ex:
+        marshal_obj = ex.submit(_compile_marshal) if marshal else None
         futs = {s: ex.submit(_compile, s, verbose, check_bounds) for s in srcs}
         objs = {s: f.result() for s, f in futs.items()}
     for s, (_, log) in objs.items():
@@ -97,6 +136,8 @@ def build(force: bool = False, verbose: bool = False, check_bounds: bool = False
         if r.returncode != 0:
             raise RuntimeError(f"link failed for {lib}:\n{r.stdout}\n{r.stderr}")
         os.replace(tmp, out)
+    if marshal:
+        _link_marshal(marshal_obj.result())
     return logs
 
 

@@ -348,3 +348,27 @@ def test_attn_tiles_per_unit_setting():
         assert b"dlm_set_attn_tiles_per_unit" in lib.dlm_last_error()
     for ok in (1, 2, 0):
         assert lib.dlm_set_attn_tiles_per_unit(ok) == 0
+
+
+def test_native_marshalling_leaves_other_forms_to_the_general_path():
+    """The native marshalling does nothing (None) for arguments that are not
+    plain CUDA tensors, Python ints or a RefineParams; the entry points then
+    raise what the general path raises."""
+    import torch
+    from paper_2608_02625_gb300 import _marshal
+    from paper_2608_02625_gb300 import binding as B
+    t = torch.zeros(2, 4)
+    i = torch.zeros(2, dtype=torch.int32)
+    prm = B.RefineParams(0.5, 1, 0.0, 7, i, i)
+    for call in (lambda: _marshal.vocab_confidence(t, i, t, t), lambda: _marshal.vocab_confidence(t, i, t),
+                 lambda: _marshal.bidir_attn(None, t, t, None, t), lambda: _marshal.attn_masked(t, t, t, i, i, 1.0, 64, t),
+                 lambda: _marshal.refine_update(i, i, i, t, object(), i, i, i),
+                 lambda: _marshal.refine_update(i, i, i, t, prm, i, i, i), lambda: _marshal.loop_launch("x", 0),
+                 lambda: _marshal.lmhead_confidence(t, t, i, t, t, [])):
+        assert call() is None
+    with pytest.raises(ValueError, match="takes CUDA tensors"):
+        B.dlm_vocab_confidence(t, i, t, t)
+    with pytest.raises(ValueError, match="takes CUDA tensors"):
+        B.dlm_refine_update(i.view(1, 2), i.view(1, 2), i.view(1, 2), t, prm, i, i, i)
+    with pytest.raises(AttributeError):
+        B.dlm_bidir_attn([1.0], t, t, None, t)
