@@ -146,3 +146,28 @@ def test_key_cache_boundary(r):
                       mask_id=case["V"], prompt=case["prompt_lens"], seqlen=case["seq_lens"])
         assert_same(gpu, ref, f"r={r} k={k}")
 
+
+
+@pytest.mark.parametrize("kind", ["distinct", "ties", "one_value", "neighbours", "signs"])
+@pytest.mark.parametrize("L", [127, 128, 129, 511, 512, 513, 2047, 2048, 2049, 8191, 8192, 8193])
+def test_register_path_edges(L, kind):
+    """The edges of the launches that hold a sequence in registers (L up to 512,
+    2048 and 8192) and the first length past them: selections that end early,
+    at the last two bits of the key, and in ties taken in index order."""
+    rng = np.random.default_rng(L)
+    B = 4
+    case = P.random_update_case(rng, B=B, L=L, V=40, ties=kind == "ties")
+    case["prompt_lens"][:2], case["seq_lens"][:2] = 0, L      # two whole sequences
+    if kind == "one_value":
+        case["conf"][:] = 0.25
+    elif kind == "neighbours":
+        case["conf"] = np.float32(0.3) + rng.integers(0, 6, (B, L)).astype(np.float32) * np.float32(2.0 ** -25)
+    elif kind == "signs":
+        case["conf"] = rng.choice(np.array([-0.0, 0.0, -1.0, 1e-40, 1.0], dtype=np.float32), (B, L))
+    for k, frac in ((1, 0.0), (L // 3, 0.0), (L - 1, 0.0), (-1, 0.1)):
+        args = dict(prompt_lens=case["prompt_lens"], seq_lens=case["seq_lens"])
+        ref = oracle.refine_update(case["tokens"], case["mask"], case["argmax"], case["conf"], edit_threshold=0.3,
+                                   remask_k=k, remask_frac=frac, mask_id=case["V"], **args)
+        gpu = run_gpu(case["tokens"], case["mask"], case["argmax"], case["conf"], tau=0.3, k=k, frac=frac,
+                      mask_id=case["V"], prompt=args["prompt_lens"], seqlen=args["seq_lens"], inplace=k == 1)
+        assert_same(gpu, ref, f"L={L} {kind} k={k}")
