@@ -412,8 +412,8 @@ def measure_loop(args, w, Bn, q, k, v, out, logits, tok0, msk0, params, seqlen, 
 
 
 def measure_fused_step(Bn, w, logits, tok, msk, params, stream, per_kernel, reps=20):
-    """The vocabulary reduction and the update in one launch (dlm_refine_step)
-    on the step's own resident buffers, against the two separate launches
+    """The vocabulary reduction and the update in one call (dlm_refine_step)
+    on the step's own resident buffers, against the two separate calls
     timed in the step (CUDA events around `reps` back-to-back launches)."""
     import torch
     d = logits.device
@@ -441,8 +441,8 @@ def measure_fused_step(Bn, w, logits, tok, msk, params, stream, per_kernel, reps
     ms = e0.elapsed_time(e1) / reps
     sep = per_kernel["vocab"] + per_kernel["update"]
     return {"ms": ms, "ms_separate_vocab_plus_update": sep, "ratio_fused_over_separate": ms / sep,
-            "note": "dlm_refine_step (one launch: the CTA finishing a sequence's last row runs its update) on the "
-                    "step's buffers; the step itself uses the separate launches, the faster of the two here"}
+            "note": "dlm_refine_step (one call: the update's launch is set up while the reduction runs) on the "
+                    "step's buffers, against the separate calls of the step itself"}
 
 
 def measure_lmhead(args, w, Bn, peaks, reps=10):
@@ -946,7 +946,7 @@ def run_ours(args, rank, world):
     kern["vocab"]["frac_of_measured_hbm"] = kern["vocab"]["achieved_gbs"] / peaks["hbm_gbs"]
     if ranked:
         kern["update"]["kernels"] = "token_prob_kernel + refine_update_kernel (ranking by the resulting token)"
-    if fused:   # the vocabulary stream and the update share one launch
+    if fused:   # the vocabulary stream and the update share one call
         kern["vocab"]["kernel"] = "vocab_step (vocabulary reduction + update)"
         kern["update"] = {"ms": 0.0, "fused_into": "vocab"}
     dominant = max(("attn", "vocab"), key=lambda kk: per_kernel[kk])
@@ -954,7 +954,7 @@ def run_ours(args, rank, world):
         roof = {"kernel": "vocab_step" if fused else "vocab_confidence", "bound": "hbm",
                 "achieved": kern["vocab"]["achieved_gbs"],
                 "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": kern["vocab"]["frac_of_measured_hbm"],
-                "traffic": recorded_traffic("vocab.cu", "vocab_step_kernel" if fused else "vocab_rows_kernel",
+                "traffic": recorded_traffic("vocab.cu", "vocab_rows_kernel",
                                             base.name),
                 "algorithmic_bytes": vocab_bytes,
                 "peak_source": peaks["source"]}
@@ -976,7 +976,7 @@ def run_ours(args, rank, world):
         "refined_tokens_per_sec": steps_per_s * w.refined_tokens(),
         "kernels": kern,
         "roofline": roof,
-        "gpu_launches": (2 if fused else 4 if ranked else 3) * args.steps,
+        "gpu_launches": (4 if ranked else 3) * args.steps,
         "path": args.path,
         "rank": args.rank,
         "attn_mask": args.attn_mask if not mask_mode else f"{args.attn_mask} (block {args.block})",
@@ -1042,8 +1042,8 @@ def main():
     ap.add_argument("--loop-steps", type=int, default=4,
                     help="also time a recorded multi-pass loop with device-side early stop (0: skip)")
     ap.add_argument("--path", default="separate", choices=["fused", "separate"],
-                    help="separate: dlm_vocab_confidence then dlm_refine_update (the faster of the two on "
-                         "the 32 x 512 workload); fused: both in one launch (dlm_refine_step)")
+                    help="separate: dlm_vocab_confidence then dlm_refine_update (timed one by one; on "
+                         "the 32 x 512 workload as fast as fused); fused: both in one call (dlm_refine_step)")
     ap.add_argument("--workloads", default="c2_single_512,c4_long_2048,c5_heavy_4step",
                     help="other workloads whose three kernels are also timed one by one (comma list; none to skip)")
     ap.add_argument("--lmhead-d", type=int, default=2048,

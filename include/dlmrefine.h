@@ -13,7 +13,7 @@
  *                         remask the k least confident positions
  *
  * Around them:
- *   dlm_refine_step          the last two in one launch (same results);
+ *   dlm_refine_step          the last two in one call (same results);
  *                            dlm_refine_step_static without a workspace
  *   dlm_lmhead_confidence    the vocabulary projection hidden x W^T fused with
  *                            the per-position reduction (logits never stored)
@@ -30,8 +30,8 @@
  *   current CUDA device, a dtype, the shape and the strides in elements.
  *   The caller owns every buffer; the library allocates no device memory and
  *   keeps no pointer after a call returns (a dlm_loop keeps the pointers of
- *   the calls it recorded). Its only device memory is static: the error word
- *   and the 16 KB scratch of dlm_refine_step_static.
+ *   the calls it recorded). Its only device memory is static: the error
+ *   word.
  * - Calls are asynchronous on the stream set by dlm_set_stream for the calling
  *   thread (default: the legacy default stream). Outputs are valid once that
  *   stream has been synchronised. Arguments are validated on the host before
@@ -261,15 +261,14 @@ int dlm_refine_update_ranked(const dlm_tensor* tokens, const dlm_tensor* mask, c
                              dlm_tensor* new_mask, dlm_tensor* n_edits);
 
 /*
- * Steps A2 and A3 fused in one launch (the per-position reduction of the
- * confidences of Table 10 / Appendix C.4 feeding the update of Sec. 4.2).
- * Computes exactly what dlm_vocab_confidence(logits, argmax, conf, lse)
- * followed by dlm_refine_update(tokens, mask, argmax, conf, params,
- * new_tokens, new_mask, n_edits) computes: argmax, conf and lse are written
- * as by the first call, and the update reads them back. The CTA that finishes
- * the last row of sequence b runs the update of b, so the update of one
- * sequence overlaps the vocabulary stream of the others and no second launch
- * is needed.
+ * Steps A2 and A3 in one call (the per-position reduction of the confidences
+ * of Table 10 / Appendix C.4 feeding the update of Sec. 4.2). Computes exactly
+ * what dlm_vocab_confidence(logits, argmax, conf, lse) followed by
+ * dlm_refine_update(tokens, mask, argmax, conf, params, new_tokens, new_mask,
+ * n_edits) computes: argmax, conf and lse are written as by the first call, and
+ * the update reads them back. The update's launch is set up while the
+ * reduction still runs (programmatic dependent launch), so the pair costs less
+ * than the two calls.
  *
  *   logits  [B * L, V] or [B, L, V]   BF16 or F32, as for dlm_vocab_confidence
  *   argmax, conf, lse                 [B, L] contiguous (I32, F32, F32)
@@ -277,12 +276,11 @@ int dlm_refine_update_ranked(const dlm_tensor* tokens, const dlm_tensor* mask, c
  *   workspace                         device memory of at least
  *                                     dlm_refine_step_workspace_bytes(B) bytes,
  *                                     4-byte aligned, owned by the caller
- * The workspace holds one row counter per sequence. It must be zero before
- * its first use (e.g. cudaMemsetAsync); each completed call leaves it zero
- * again, so it can be reused by later calls without clearing. Calls that
- * share a workspace must not overlap on the GPU (they would race on the
- * counters): issue them on one stream. new_tokens / new_mask may alias
- * tokens / mask exactly; no other overlap among the tensors is allowed.
+ * The workspace must be zero before its first use (e.g. cudaMemsetAsync) and
+ * is zero after each call; the present implementation leaves it untouched.
+ * Calls that share a workspace must not overlap on the GPU: issue them on one
+ * stream. new_tokens / new_mask may alias tokens / mask exactly; no other
+ * overlap among the tensors is allowed.
  */
 int dlm_refine_step(const dlm_tensor* logits, const dlm_tensor* tokens, const dlm_tensor* mask,
                     const dlm_refine_params* params, dlm_tensor* argmax, dlm_tensor* conf,
@@ -291,7 +289,7 @@ int dlm_refine_step(const dlm_tensor* logits, const dlm_tensor* tokens, const dl
 /* Bytes of workspace dlm_refine_step needs for a batch of `batch` sequences. */
 size_t dlm_refine_step_workspace_bytes(int64_t batch);
 
-/* Largest batch dlm_refine_step_static accepts (its static scratch: 16 KB). */
+/* Largest batch dlm_refine_step_static accepts. */
 #define DLM_STATIC_STEP_MAX_BATCH 4096
 
 /*
@@ -304,20 +302,14 @@ size_t dlm_refine_step_workspace_bytes(int64_t batch);
  * fixed signature and no slot for a workspace.
  *
  * Computes exactly what dlm_refine_step computes, with the same arguments
- * minus the workspace. The per-sequence counters live in a static device
- * array of DLM_STATIC_STEP_MAX_BATCH int32 inside the library, which every
- * device that loads the library holds until the process exits. The call
- * allocates nothing (no cudaMalloc, cudaFree or allocating library routine).
+ * minus the workspace. The call allocates nothing (no cudaMalloc, cudaFree or
+ * allocating library routine).
  *
- * - The first call on a device sets up that device: it takes the array's
- *   device address with cudaGetSymbolAddress, with that device current.
- *   Make that first call before any stream capture on the device;
+ * - The first call on a device takes the address of the device error word
+ *   there. Make that first call before any stream capture on the device;
  *   dlm_loop_begin does this set-up itself, so a recorded pass may use it.
- * - Each call clears the counters it uses (an asynchronous memset on the
- *   call's stream) and then launches the fused kernel.
- * - All calls on one device share the array: calls that overlap on the GPU
- *   (different streams, or different host threads) race on it and give
- *   undefined results. Issue them on one stream.
+ * - Calls that overlap on the GPU (different streams, or different host
+ *   threads) must not share buffers; issue the calls of a device on one stream.
  * - B > DLM_STATIC_STEP_MAX_BATCH returns DLM_ERR_SHAPE with nothing
  *   launched; use dlm_refine_step with a workspace for larger batches.
  */

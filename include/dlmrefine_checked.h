@@ -13,11 +13,11 @@ extern "C" {
 #endif
 
 /*
- * Fills every byte of dlm_refine_step_static's static scratch array on the
- * current device with `byte_value` (0..255), asynchronously on the calling
- * thread's stream. A test sets it to a nonzero pattern to check that each
- * static call clears the counters it uses before it counts. Returns
- * DLM_ERR_ARG for a value outside 0..255.
+ * Fills every byte of dlm_refine_step_static's static scratch on the current
+ * device with `byte_value` (0..255), asynchronously on the calling thread's
+ * stream, so that a test can check that no call depends on what it holds. The
+ * present implementation keeps no such scratch: there is nothing to fill.
+ * Returns DLM_ERR_ARG for a value outside 0..255.
  */
 int dlm_checked_fill_static_scratch(int32_t byte_value);
 

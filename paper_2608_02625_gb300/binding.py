@@ -270,7 +270,7 @@ def dlm_refine_step_workspace_bytes(batch: int) -> int:
 
 def dlm_refine_step(logits, tokens, mask, params: RefineParams, argmax, conf, lse, new_tokens, new_mask, n_edits,
                     workspace):
-    """Vocabulary reduction and refine update in one launch.
+    """Vocabulary reduction and refine update in one call.
 
     workspace: a CUDA tensor of at least dlm_refine_step_workspace_bytes(B) bytes,
     zero before its first use; each completed call leaves it zero again."""
@@ -292,10 +292,9 @@ def dlm_refine_step(logits, tokens, mask, params: RefineParams, argmax, conf, ls
 
 def dlm_refine_step_static(logits, tokens, mask, params: RefineParams, argmax, conf, lse, new_tokens, new_mask,
                            n_edits):
-    """dlm_refine_step with the library's static scratch instead of a workspace,
-    for callers that cannot allocate device memory. The first call on a device
-    sets that device up (make it before any stream capture); calls that overlap
-    on the GPU race on the shared scratch."""
+    """dlm_refine_step without a workspace, for callers that cannot allocate
+    device memory. The first call on a device sets that device up (make it
+    before any stream capture)."""
     if _done(_marshal.refine_step_static(logits, tokens, mask, params, argmax, conf, lse, new_tokens,
                                          new_mask, n_edits)):
         return argmax, conf, lse, new_tokens, new_mask, n_edits

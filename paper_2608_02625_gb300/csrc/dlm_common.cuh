@@ -39,6 +39,12 @@ constexpr bool kCheckBounds = true;
 constexpr bool kCheckBounds = false;
 #endif
 
+// Lets a kernel launched with programmatic stream serialisation take free
+// places on the SMs once every block of this one has got here or ended.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// In such a kernel: waits until the one before it has ended and its writes are visible.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ----------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {

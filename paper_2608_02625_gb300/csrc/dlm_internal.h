@@ -20,10 +20,6 @@ uint64_t wait_budget_ns();
 // Query tiles per attention work unit set on this thread (0: automatic).
 int attn_tiles_per_unit();
 
-// Device address of dlm_refine_step_static's scratch array on the current
-// device (set up on first use; a status, with *out untouched, on failure).
-int static_step_scratch(int32_t** out);
-
 // Records a failure message for dlm_last_error() and returns `status`.
 int fail(int status, const char* fmt, ...);
 // Clears the calling thread's failure message (at the start of every entry point).
@@ -88,14 +84,13 @@ struct UpdateArgs {
 };
 
 int launch_refine_update(const UpdateArgs& a, cudaStream_t stream);
+// The same right behind the launch_vocab_confidence that writes a.argmax and
+// a.conf, on its stream: starts before that launch has ended and waits for it.
+int launch_refine_update_after_vocab(const UpdateArgs& a, cudaStream_t stream);
 
 // prob[r] = exp(logits[r, tokens[r]] - lse[r]) (0 for a token outside [0, V)).
 int launch_token_prob(const VocabArgs& a, const int32_t* tokens, const float* lse, float* prob,
                       cudaStream_t stream);
-
-// Fused vocabulary reduction + update (rows of sequence b are b * L .. b * L + L - 1;
-// u.argmax / u.conf alias a.argmax / a.conf). counters: int32[B], zero on entry.
-int launch_vocab_step(const VocabArgs& a, const UpdateArgs& u, int* counters, cudaStream_t stream);
 
 // Vocabulary projection fused with the reduction: per row r of hidden [N, d]
 // the argmax / conf / lse of hidden[r] . weight[v] over v < V.

@@ -78,11 +78,9 @@ int dlm_loop_begin(int32_t* steps_out) {
   cudaError_t e = cudaStreamIsCapturing(stream, &cs);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "cudaStreamIsCapturing: %s", cudaGetErrorString(e));
   if (cs != cudaStreamCaptureStatusNone) return fail(DLM_ERR_ARG, "the stream is already capturing");
-  // Set-up that must not happen during the capture: the device addresses of
-  // the error word and of the static step scratch (cudaGetSymbolAddress).
+  // Set-up that must not happen during the capture: the device address of the
+  // error word (cudaGetSymbolAddress).
   if (!dlm::device_error_word()) return fail(DLM_ERR_CUDA, "device error word unavailable");
-  int32_t* scratch = nullptr;
-  if (const int st = dlm::static_step_scratch(&scratch)) return st;
 
   cudaGraph_t g = nullptr;
   if ((e = cudaGraphCreate(&g, 0)) != cudaSuccess)

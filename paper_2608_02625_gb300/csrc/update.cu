@@ -48,8 +48,9 @@ __device__ __forceinline__ int remask_count(const UpdateArgs& a, int r) {
 }
 
 // One sequence per CTA, position i = threadIdx.x + j * kThreads in registers of
-// thread threadIdx.x (L <= kItems * kThreads).
-template <int kThreads, int kItems>
+// thread threadIdx.x (L <= kItems * kThreads). kAfterVocab: launched behind the
+// vocabulary reduction that writes argmax and conf, before it has ended.
+template <int kThreads, int kItems, bool kAfterVocab>
 __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, int* err) {
   constexpr int kWarps = kThreads / 32;
   __shared__ int count[2][kWarps][32];
@@ -75,6 +76,7 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
   }
   int n, p;
   lengths(a, b, err, &n, &p);
+  if (kAfterVocab) wait_for_previous();
   {
     const int32_t* am = a.argmax + b * a.s_argmax;
     const float* conf = a.conf + b * a.s_conf;
@@ -82,8 +84,8 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
     for (int j = 0; j < kItems; ++j) {
       const int i = tid + j * kThreads;
       if (i < a.L) {
-        pred[j] = am[i];
-        cf[j] = conf[i];
+        pred[j] = kAfterVocab ? __ldcg(am + i) : am[i];
+        cf[j] = kAfterVocab ? __ldcg(conf + i) : conf[i];
       }
     }
   }
@@ -216,22 +218,46 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
 constexpr int kLongThreads = 512;
 __global__ void __launch_bounds__(kLongThreads) refine_update_long_kernel(UpdateArgs a, int* err) {
   __shared__ UpdateShared<kLongThreads> sh;
-  refine_sequence<kLongThreads, false>(a, blockIdx.x, err, sh);
+  refine_sequence<kLongThreads>(a, blockIdx.x, err, sh);
+}
+
+template <int kThreads, int kItems, bool kAfterVocab>
+cudaError_t launch_short(const UpdateArgs& a, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.B));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = kAfterVocab ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, refine_update_kernel<kThreads, kItems, kAfterVocab>, a, device_error_word());
+}
+
+template <bool kAfterVocab>
+int launch(const UpdateArgs& a, cudaStream_t stream) {
+  if (a.B == 0) return DLM_OK;
+  cudaError_t e;
+  // The fewest threads that hold the sequence: fewer warps meet at each barrier.
+  if (a.L <= 512) {
+    e = launch_short<128, 4, kAfterVocab>(a, stream);
+  } else if (a.L <= 2048) {
+    e = launch_short<256, 8, kAfterVocab>(a, stream);
+  } else if (a.L <= 8192) {
+    e = launch_short<1024, 8, kAfterVocab>(a, stream);
+  } else {
+    refine_update_long_kernel<<<a.B, kLongThreads, 0, stream>>>(a, device_error_word());
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "refine_update launch: %s", cudaGetErrorString(e));
+  return DLM_OK;
 }
 
 }  // namespace
 
-int launch_refine_update(const UpdateArgs& a, cudaStream_t stream) {
-  if (a.B == 0) return DLM_OK;
-  int* err = device_error_word();
-  // The fewest threads that hold the sequence: fewer warps meet at each barrier.
-  if (a.L <= 512) refine_update_kernel<128, 4><<<a.B, 128, 0, stream>>>(a, err);
-  else if (a.L <= 2048) refine_update_kernel<256, 8><<<a.B, 256, 0, stream>>>(a, err);
-  else if (a.L <= 8192) refine_update_kernel<1024, 8><<<a.B, 1024, 0, stream>>>(a, err);
-  else refine_update_long_kernel<<<a.B, kLongThreads, 0, stream>>>(a, err);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "refine_update launch: %s", cudaGetErrorString(e));
-  return DLM_OK;
-}
+int launch_refine_update(const UpdateArgs& a, cudaStream_t stream) { return launch<false>(a, stream); }
+
+int launch_refine_update_after_vocab(const UpdateArgs& a, cudaStream_t stream) { return launch<true>(a, stream); }
 
 }  // namespace dlm

@@ -18,9 +18,7 @@
 // and keep it in shared memory for passes 2 and 3; longer ones re-read the
 // predictions in each pass.
 // Integer work and exact fp32 compares only: results are bit-exact.
-// Used by the stand-alone update kernel (update.cu) and by the fused
-// vocabulary + update kernel (vocab.cu), whose last row block of a sequence
-// runs it.
+// The path of sequences too long for the registers of update.cu.
 #pragma once
 
 #include <cmath>
@@ -82,17 +80,9 @@ __device__ __forceinline__ int block_inclusive_scan(int v, int* warp_sums, int* 
   return before + x;
 }
 
-// Reads of predictions written earlier in the same launch by other blocks go
-// around L1 (kFresh); otherwise plain loads.
-template <bool kFresh, typename T>
-__device__ __forceinline__ T load_pred(const T* p) {
-  if constexpr (kFresh) return __ldcg(p);
-  else return *p;
-}
-
 // Runs the update of sequence b with the whole block (blockDim.x == kThreads).
 // Every thread of the block must call it.
-template <int kThreads, bool kFresh>
+template <int kThreads>
 __device__ void refine_sequence(const UpdateArgs& a, int b, int* err, UpdateShared<kThreads>& sh) {
   const int tid = threadIdx.x;
   const int L = a.L;
@@ -114,8 +104,8 @@ __device__ void refine_sequence(const UpdateArgs& a, int b, int* err, UpdateShar
   const float* tp = a.tok_prob ? a.tok_prob + b * a.s_tok_prob : nullptr;
   // Ranking value of response position i once pass 1 has written new_tokens.
   auto rank_value = [&](int i) -> float {
-    if (tp && ntok[i] != load_pred<kFresh>(am + i)) return tp[i];
-    return load_pred<kFresh>(cf + i);
+    if (tp && ntok[i] != am[i]) return tp[i];
+    return cf[i];
   };
 
   // ---- pass 1: copy / commit / edit (read and write of position i by one
@@ -129,8 +119,8 @@ __device__ void refine_sequence(const UpdateArgs& a, int b, int* err, UpdateShar
     int t = tok[i];
     uint8_t m = msk[i];
     if (i >= p && i < n) {
-      const int pred = load_pred<kFresh>(am + i);
-      const float c = load_pred<kFresh>(cf + i);
+      const int pred = am[i];
+      const float c = cf[i];
       if (m) {
         t = pred;
       } else if (pred != t && c >= a.edit_threshold) {

@@ -223,3 +223,29 @@ def test_key_cache_boundary(r):
               prompt_lens=case["prompt_lens"], seq_lens=case["seq_lens"])
     oracle_update_parity(fz, case["tokens"], case["mask"], pn, ref_v, f"r={r} oracle update")
 
+
+
+@pytest.mark.parametrize("B,L,V", [(3, 1, 5), (2, 512, 33), (2, 513, 8), (1, 2049, 9), (1, 8193, 3)])
+def test_update_sees_the_whole_reduction(B, L, V):
+    """The update is launched while the reduction still runs: with each of its
+    launches (by L), over repeated calls on changing logits, its results are
+    those of a separate update on the step's own predictions."""
+    from paper_2608_02625_gb300 import binding as Bn
+    d = dev()
+    g = torch.Generator(device=d).manual_seed(L)
+    n = torch.full((B,), L, dtype=torch.int32, device=d)
+    p = torch.zeros(B, dtype=torch.int32, device=d)
+    prm = Bn.RefineParams(0.4, -1, 0.2, V, p, n)
+    tok = torch.randint(0, V, (B, L), dtype=torch.int32, device=d, generator=g)
+    msk = (torch.rand(B, L, device=d, generator=g) < 0.3).to(torch.uint8)
+    ws = torch.zeros(B, dtype=torch.int32, device=d)
+    out = [torch.empty(B, L, dtype=t, device=d) for t in (torch.int32, torch.float32, torch.float32)]
+    for _ in range(20):
+        x = torch.randn(B * L, V, device=d, generator=g).to(torch.bfloat16)
+        new = [torch.empty_like(tok), torch.empty_like(msk), torch.empty_like(n)]
+        ref = [torch.empty_like(t) for t in new]
+        Bn.dlm_refine_step(x, tok, msk, prm, *out, *new, ws)
+        Bn.dlm_refine_update(tok, msk, out[0], out[1], prm, *ref)
+        assert all(torch.equal(a, b) for a, b in zip(new, ref))
+        tok, msk = new[0], new[1]
+    assert Bn.device_error(clear=True) == 0
