@@ -6,16 +6,18 @@
 //   S = sum exp(x - m),  lse = m + ln S,  conf = 1 / S  (= exp(m - lse)).
 //
 // An HBM-bound stream: every logit is read exactly once, 16 bytes per load,
-// coalesced across the block; with several waves of rows the loads go through
-// a per-thread shared-memory staging ring (cp.async, eight vectors in flight
-// per thread), otherwise straight into registers (four in flight). Each thread
-// keeps an online (max, first index, scaled sum) triple; the sum is rescaled
-// only when a 16-byte vector raises the running maximum, and the exponentials
-// go two at a time through the packed fp32 FMA and add of the sm_100 family,
-// so that the instruction stream stays below what HBM delivers per SM.
-// Threads combine by warp shuffles, warps through shared memory, and -- with
-// at most two rows per SM -- the CTAs of a thread-block cluster that split one
-// row combine through distributed shared memory (no global scratch memory).
+// coalesced across the threads of a row; what lies before a row's first
+// 16-byte boundary and after its last (rows packed under an odd vocabulary
+// start anywhere) is loaded one element per thread beside the stream. Each
+// thread keeps an online (max, first index, scaled sum) triple; the sum is
+// rescaled only when a 16-byte vector raises the running maximum, and the
+// exponentials go two at a time through the packed fp32 FMA and add of the
+// sm_100 family, so that the instruction stream stays below what HBM delivers
+// per SM. (Rows off 16-byte boundaries took scalar loads throughout before:
+// 512 rows of 151553 bf16 94.5 us, now 27.8, as long as rows of 151552.)
+// Who works on a row depends on its length and on how many there are
+// (launch_typed): a warp, a CTA, or a thread-block cluster whose warps' parts
+// meet in one CTA through distributed shared memory (no global scratch).
 #include <cooperative_groups.h>
 
 #include <cmath>
@@ -30,7 +32,7 @@ namespace dlm {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kUnroll = 4;
+constexpr int kWarps = kThreads / 32;
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct Partial {
@@ -39,20 +41,34 @@ struct Partial {
   float s;    // sum of exp(x - m)
 };
 
-// Combines two partials; the lower index wins ties of the maximum.
+// Order-preserving map of fp32 to int (-0 below +0).
+__device__ __forceinline__ int order_key(float x) {
+  const int i = __float_as_int(x);
+  return i ^ ((i >> 31) & 0x7FFFFFFF);
+}
+
+// Combines two partials; the lower index wins equal maxima.
 __device__ __forceinline__ Partial combine(Partial a, Partial b) {
   Partial r;
   r.m = fmaxf(a.m, b.m);
-  if (a.m > b.m) r.idx = a.idx;
-  else if (b.m > a.m) r.idx = b.idx;
-  else r.idx = min(a.idx, b.idx);
-  if (r.m == -INFINITY) {
-    r.s = 0.f;
-  } else {
-    float sa = a.m == -INFINITY ? 0.f : a.s * ex2_approx((a.m - r.m) * kLog2e);
-    float sb = b.m == -INFINITY ? 0.f : b.s * ex2_approx((b.m - r.m) * kLog2e);
-    r.s = sa + sb;
-  }
+  r.idx = a.m > b.m ? a.idx : b.m > a.m ? b.idx : min(a.idx, b.idx);
+  r.s = a.s * (a.m == -INFINITY ? 0.f : ex2_approx((a.m - r.m) * kLog2e)) +
+        b.s * (b.m == -INFINITY ? 0.f : ex2_approx((b.m - r.m) * kLog2e));
+  return r;
+}
+
+// The warp's partials as one, in every lane; the lower index wins equal maxima.
+// One reduction each for the maximum and the index, then the rescaled sums.
+template <int kLanes = 32>
+__device__ __forceinline__ Partial warp_reduce(Partial p) {
+  const int k = __reduce_max_sync(0xffffffffu, order_key(p.m));
+  Partial r;
+  r.m = __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF));
+  r.idx = __reduce_min_sync(0xffffffffu, p.m == r.m ? p.idx : 0x7FFFFFFF);
+  // A partial without a finite entry has sum 0 (or NaN, which must stay).
+  r.s = p.s * (p.m == -INFINITY ? 0.f : ex2_approx((p.m - r.m) * kLog2e));
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) r.s += __shfl_xor_sync(0xffffffffu, r.s, o);
   return r;
 }
 
@@ -99,16 +115,17 @@ struct Vec<false> {
   }
 };
 
-// Folds one value x at element index e into p (the scalar path: rows whose
-// length or alignment rules out 16-byte vectors, and a row's ragged tail).
-__device__ __forceinline__ void fold1(Partial& p, float& mL, float x, int e) {
+// Folds one value x at element index e into p, in any order of the indices
+// (a row's elements outside its vectors).
+__device__ __forceinline__ void fold_edge(Partial& p, float x, int e) {
   if (x > p.m) {
-    p.s = (p.m == -INFINITY) ? 0.f : p.s * ex2_approx((p.m - x) * kLog2e);
+    p.s = p.s * (p.m == -INFINITY ? 0.f : ex2_approx((p.m - x) * kLog2e)) + 1.f;
     p.m = x;
     p.idx = e;
-    mL = x * kLog2e;
+  } else if (x != -INFINITY) {
+    p.s += ex2_approx((x - p.m) * kLog2e);  // NaN stays NaN
+    if (x == p.m) p.idx = min(p.idx, e);
   }
-  if (p.m != -INFINITY) p.s += ex2_approx(fmaf(x, kLog2e, -mL));
 }
 
 // Folds one 16-byte vector of kN values starting at element index e0: the
@@ -141,69 +158,85 @@ __device__ __forceinline__ void fold_vec(Partial& p, float& mL, float2& s2, cons
   }
 }
 
-// Reduces the block's partials into thread 0's return value.
+// Reduces the block's partials into warp 0's return value.
 __device__ __forceinline__ Partial block_reduce(Partial p) {
-  __shared__ Partial warp_part[kThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Partial q;
-    q.m = __shfl_xor_sync(0xffffffffu, p.m, o);
-    q.idx = __shfl_xor_sync(0xffffffffu, p.idx, o);
-    q.s = __shfl_xor_sync(0xffffffffu, p.s, o);
-    p = combine(p, q);
-  }
+  __shared__ Partial warp_part[kWarps];
+  p = warp_reduce(p);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) warp_part[warp] = p;
   __syncthreads();
   if (warp == 0) {
-    p = lane < kThreads / 32 ? warp_part[lane] : Partial{-INFINITY, 0x7FFFFFFF, 0.f};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      Partial q;
-      q.m = __shfl_xor_sync(0xffffffffu, p.m, o);
-      q.idx = __shfl_xor_sync(0xffffffffu, p.idx, o);
-      q.s = __shfl_xor_sync(0xffffffffu, p.s, o);
-      p = combine(p, q);
-    }
+    p = lane < kWarps ? warp_part[lane] : Partial{-INFINITY, 0x7FFFFFFF, 0.f};
+    p = warp_reduce<kWarps>(p);
   }
   return p;
 }
 
-// Scans elements [e_begin, e_end) of one row.
-template <bool BF16, bool VEC>
-__device__ __forceinline__ Partial scan_range(const char* row, int64_t e_begin, int64_t e_end) {
+// A row of V elements as a run of whole 16-byte vectors with up to kN - 1
+// elements before and after it.
+template <bool BF16>
+struct Row {
+  const char* base;
+  const uint4* vec;  // first vector: element `head`
+  int64_t nvec;
+  int head, tail;
+  __device__ __forceinline__ Row(const VocabArgs& a, int64_t r) {
+    constexpr int kEsz = BF16 ? 2 : 4, kN = 16 / kEsz;
+    base = static_cast<const char*>(a.logits) + r * a.row_stride * kEsz;
+    const int64_t before = static_cast<int64_t>((0 - reinterpret_cast<uintptr_t>(base)) & 15u) / kEsz;
+    head = static_cast<int>(before < a.V ? before : a.V);
+    vec = reinterpret_cast<const uint4*>(base + head * kEsz);
+    nvec = (a.V - head) / kN;
+    tail = static_cast<int>(a.V - head - nvec * kN);
+  }
+};
+
+// The element outside the row's vectors that thread t of a row's threads owns:
+// t < 8 before them, 8 <= t < 16 after them (-inf where there is none).
+template <bool BF16>
+__device__ __forceinline__ float load_edge(const Row<BF16>& row, int t, bool first, bool last, int64_t V, int* e) {
+  *e = t < 8 ? t : static_cast<int>(V) - row.tail + t - 8;
+  const bool mine = t < 8 ? first && t < row.head : last && t < 8 + row.tail;
+  return mine ? Vec<BF16>::load1(row.base, *e) : -INFINITY;
+}
+
+// Scans vectors [v_begin, v_end) of a row with kWidth threads, of which this
+// is number t, kUnroll loads in flight.
+template <bool BF16, int kWidth, int kUnroll>
+__device__ __forceinline__ Partial scan_vectors(const Row<BF16>& row, int64_t v_begin, int64_t v_end, int t) {
   using VT = Vec<BF16>;
   constexpr int kN = VT::kN;
   Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
   float mL = 0.f;
-  if constexpr (VEC) {
-    // e_begin and e_end are multiples of kN except possibly the row's end.
-    const int64_t v_begin = e_begin / kN;
-    const int64_t v_end = e_end / kN;  // full vectors
-    const uint4* vp = reinterpret_cast<const uint4*>(row);
-    float2 s2 = make_float2(0.f, 0.f);
-    int64_t vi = v_begin + threadIdx.x;
-    for (; vi + (kUnroll - 1) * kThreads < v_end; vi += kUnroll * kThreads) {
-      uint4 raw[kUnroll];
+  float2 s2 = make_float2(0.f, 0.f);
+  int64_t vi = v_begin + t;
+  for (; vi + (kUnroll - 1) * kWidth < v_end; vi += kUnroll * kWidth) {
+    uint4 raw[kUnroll];
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) raw[u] = ld_stream16(vp + vi + u * kThreads);
+    for (int u = 0; u < kUnroll; ++u) raw[u] = ld_stream16(row.vec + vi + u * kWidth);
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < kUnroll; ++u) {
+      float x[kN];
+      VT::unpack(raw[u], x);
+      fold_vec<kN>(p, mL, s2, x, row.head + static_cast<int>((vi + u * kWidth) * kN));
+    }
+  }
+  // The last, partial round: its loads in flight together too.
+  if (vi < v_end) {
+    uint4 raw[kUnroll - 1];
+#pragma unroll
+    for (int u = 0; u < kUnroll - 1; ++u)
+      if (vi + u * kWidth < v_end) raw[u] = ld_stream16(row.vec + vi + u * kWidth);
+#pragma unroll
+    for (int u = 0; u < kUnroll - 1; ++u) {
+      if (vi + u * kWidth < v_end) {
         float x[kN];
         VT::unpack(raw[u], x);
-        fold_vec<kN>(p, mL, s2, x, static_cast<int>((vi + u * kThreads) * kN));
+        fold_vec<kN>(p, mL, s2, x, row.head + static_cast<int>((vi + u * kWidth) * kN));
       }
     }
-    for (; vi < v_end; vi += kThreads) {
-      float x[kN];
-      VT::unpack(ld_stream16(vp + vi), x);
-      fold_vec<kN>(p, mL, s2, x, static_cast<int>(vi * kN));
-    }
-    p.s = s2.x + s2.y;
-    e_begin = v_end * kN;  // scalar tail (row length not a multiple of kN)
   }
-  for (int64_t e = e_begin + threadIdx.x; e < e_end; e += kThreads)
-    fold1(p, mL, VT::load1(row, e), static_cast<int>(e));
+  p.s = s2.x + s2.y;
   return p;
 }
 
@@ -223,43 +256,39 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// scan_range for 16-byte aligned rows with the loads staged through shared
+// scan_vectors of a whole row by a block with the loads staged through shared
 // memory: each thread keeps kStages of its vectors in flight in its own slots
 // of `ring` ([kStages][kThreads]), reads back only what it copied itself (so
 // no block barrier), and refills a slot as soon as its value is in registers:
 // twice the bytes in flight of the register-loaded scan, with no registers
 // held for them.
 template <bool BF16, int kStages>
-__device__ __forceinline__ Partial scan_range_staged(const char* row, int64_t e_begin, int64_t e_end, uint4* ring) {
+__device__ __forceinline__ Partial scan_row_staged(const Row<BF16>& row, uint4* ring) {
   using VT = Vec<BF16>;
   constexpr int kN = VT::kN;
   Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
   float mL = 0.f;
   float2 s2 = make_float2(0.f, 0.f);
-  const uint4* vp = reinterpret_cast<const uint4*>(row);
-  const int64_t v_end = e_end / kN;
-  const int64_t first = e_begin / kN + threadIdx.x;
-  const int nk = first < v_end ? static_cast<int>((v_end - first + kThreads - 1) / kThreads) : 0;
+  const int64_t first = threadIdx.x;
+  const int nk = first < row.nvec ? static_cast<int>((row.nvec - first + kThreads - 1) / kThreads) : 0;
   uint4* mine = ring + threadIdx.x;
 #pragma unroll
   for (int k = 0; k < kStages; ++k) {
-    if (k < nk) cp_async16(mine + k * kThreads, vp + first + static_cast<int64_t>(k) * kThreads);
+    if (k < nk) cp_async16(mine + k * kThreads, row.vec + first + static_cast<int64_t>(k) * kThreads);
     cp_async_commit();
   }
   for (int k = 0; k < nk; ++k) {
     cp_async_wait<kStages - 1>();  // the group of vector k has landed
     uint4* slot = mine + (k % kStages) * kThreads;
     const uint4 v = *slot;
-    if (k + kStages < nk) cp_async16_after(slot, vp + first + static_cast<int64_t>(k + kStages) * kThreads, v.w);
+    if (k + kStages < nk) cp_async16_after(slot, row.vec + first + static_cast<int64_t>(k + kStages) * kThreads, v.w);
     cp_async_commit();
     float x[kN];
     VT::unpack(v, x);
-    fold_vec<kN>(p, mL, s2, x, static_cast<int>((first + static_cast<int64_t>(k) * kThreads) * kN));
+    fold_vec<kN>(p, mL, s2, x, row.head + static_cast<int>((first + static_cast<int64_t>(k) * kThreads) * kN));
   }
   cp_async_wait<0>();
   p.s = s2.x + s2.y;
-  for (int64_t e = v_end * kN + threadIdx.x; e < e_end; e += kThreads)  // ragged tail
-    fold1(p, mL, VT::load1(row, e), static_cast<int>(e));
   return p;
 }
 
@@ -272,68 +301,84 @@ __device__ __forceinline__ void write_out(const VocabArgs& a, int64_t rowi, Part
 }
 
 // One CTA per row (grid-stride over rows). kStaged: the loads go through the
-// shared-memory staging ring of scan_range_staged (16-byte aligned rows only).
+// shared-memory staging ring of scan_row_staged.
 constexpr int kStages = 8;
-template <bool BF16, bool VEC, bool kStaged>
+template <bool BF16, bool kStaged>
 __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
   __shared__ uint4 ring[kStaged ? kStages * kThreads : 1];
   launch_dependents();
-  const int esz = BF16 ? 2 : 4;
   for (int64_t rowi = blockIdx.x; rowi < a.N; rowi += gridDim.x) {
-    const char* row = static_cast<const char*>(a.logits) + rowi * a.row_stride * esz;
-    Partial p = kStaged ? scan_range_staged<BF16, kStages>(row, 0, a.V, ring) : scan_range<BF16, VEC>(row, 0, a.V);
+    const Row<BF16> row(a, rowi);
+    int e;
+    const float edge = load_edge(row, threadIdx.x, true, true, a.V, &e);
+    Partial p = kStaged ? scan_row_staged<BF16, kStages>(row, ring) : scan_vectors<BF16, kThreads, 4>(row, 0, row.nvec, threadIdx.x);
+    fold_edge(p, edge, e);
     p = block_reduce(p);
     if (threadIdx.x == 0) write_out(a, rowi, p);
     __syncthreads();
   }
 }
 
-// Rows split over a cluster of `csize` CTAs: CTA c of a cluster scans chunk c
-// of the row, rank 0 combines the chunk partials through distributed shared
-// memory. Persistent: cluster k takes rows k, k + clusters, ..., so a launch is
-// one wave of resident CTAs, with no per-row launch and ramp-up; the partial
-// slots alternate between rows, so one cluster barrier per row suffices (rank
-// 0 reads row i's partials before it scans row i + 1, whose barrier the other
-// CTAs must pass before they overwrite that slot with row i + 2's).
-template <bool BF16, bool VEC>
-__global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a) {
-  __shared__ Partial cta_part[2];
+// One warp per row: many short rows.
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads, 4) vocab_short_rows_kernel(VocabArgs a) {
   launch_dependents();
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * kWarps;
+  for (int64_t rowi = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5); rowi < a.N; rowi += warps) {
+    const Row<BF16> row(a, rowi);
+    int e;
+    const float edge = load_edge(row, lane, true, true, a.V, &e);
+    Partial p = scan_vectors<BF16, 32, 4>(row, 0, row.nvec, lane);
+    fold_edge(p, edge, e);
+    p = warp_reduce(p);
+    if (lane == 0) write_out(a, rowi, p);
+  }
+}
+
+// Rows split over a cluster of `csize` CTAs: CTA c scans chunk c of the row,
+// every warp stores its part in rank 0's shared memory, and one warp of rank 0
+// combines them. Persistent: cluster k takes rows k, k + clusters, ..., so a
+// launch is one wave of resident CTAs, with no per-row launch and ramp-up; the
+// slots alternate between rows, so one cluster barrier per row suffices (rank
+// 0 reads row i's parts before it scans row i + 1, whose barrier the other
+// CTAs must pass before they overwrite that slot with row i + 2's).
+constexpr int kMaxCluster = 16;
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a) {
+  __shared__ Partial parts[2][kMaxCluster * kWarps];
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = static_cast<int>(cluster.num_blocks());
   const int crank = static_cast<int>(cluster.block_rank());
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nclusters = gridDim.x / csize;
-  const int esz = BF16 ? 2 : 4;
-  const int kN = BF16 ? 8 : 4;
-  // Chunk boundaries on whole vectors.
-  const int64_t nvec = (a.V + kN - 1) / kN;
-  const int64_t per = (nvec + csize - 1) / csize;
-  int64_t e0 = crank * per * kN;
-  int64_t e1 = (crank + 1) * per * kN;
-  if (e0 > a.V) e0 = a.V;
-  if (e1 > a.V) e1 = a.V;
+  launch_dependents();
+  cluster.barrier_arrive();  // rank 0's shared memory may be written once every CTA runs
   int it = 0;
   for (int64_t rowi = blockIdx.x / csize; rowi < a.N; rowi += nclusters, ++it) {
-    const char* row = static_cast<const char*>(a.logits) + rowi * a.row_stride * esz;
-    Partial p = scan_range<BF16, VEC>(row, e0, e1);
-    p = block_reduce(p);
-    if (threadIdx.x == 0) cta_part[it & 1] = p;
+    const Row<BF16> row(a, rowi);
+    const int64_t per = (row.nvec + csize - 1) / csize;
+    const int64_t v0 = crank * per < row.nvec ? crank * per : row.nvec;
+    const int64_t v1 = v0 + per < row.nvec ? v0 + per : row.nvec;
+    int e;
+    const float edge = load_edge(row, threadIdx.x, crank == 0, crank == csize - 1, a.V, &e);
+    Partial p = scan_vectors<BF16, kThreads, 4>(row, v0, v1, threadIdx.x);
+    fold_edge(p, edge, e);
+    p = warp_reduce(p);
+    if (it == 0) cluster.barrier_wait();
+    if (lane == 0) *cluster.map_shared_rank(&parts[it & 1][crank * kWarps + warp], 0) = p;
     cluster.sync();
-    if (crank == 0 && threadIdx.x < 32) {
+    if (crank == 0 && warp == 0) {
+      const int n = csize * kWarps;
       Partial q{-INFINITY, 0x7FFFFFFF, 0.f};
-      if (static_cast<int>(threadIdx.x) < csize) q = *cluster.map_shared_rank(&cta_part[it & 1], threadIdx.x);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        Partial t;
-        t.m = __shfl_xor_sync(0xffffffffu, q.m, o);
-        t.idx = __shfl_xor_sync(0xffffffffu, q.idx, o);
-        t.s = __shfl_xor_sync(0xffffffffu, q.s, o);
-        q = combine(q, t);
-      }
-      if (threadIdx.x == 0) write_out(a, rowi, q);
+      for (int j = 0; j < kMaxCluster * kWarps; j += 32)
+        if (j + lane < n) q = combine(q, parts[it & 1][j + lane]);
+      q = warp_reduce(q);
+      if (lane == 0) write_out(a, rowi, q);
     }
   }
-  cluster.sync();  // keep every CTA's shared memory alive until rank 0 has read it
+  if (it == 0) cluster.barrier_wait();
 }
 
 // Probability of a given token of each row: one gathered logit per row.
@@ -354,70 +399,62 @@ __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int3
   prob[r] = p;
 }
 
-template <bool BF16, bool VEC>
+// One wave of clusters of (at most) `csize` CTAs, each taking rows in turn.
+template <bool BF16>
+int launch_cluster(const VocabArgs& a, int csize, cudaStream_t stream) {
+  const auto kernel = vocab_cluster_kernel<BF16>;
+  int active = 0;
+  while ((active = active_clusters(reinterpret_cast<const void*>(kernel), csize, kThreads, 0)) == 0 && csize > 1) csize /= 2;
+  if (active == 0) return fail(DLM_ERR_CUDA, "vocab_confidence: no cluster launch fits the device");
+  const int64_t nclusters = a.N < active ? a.N : active;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(nclusters * csize));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence cluster launch: %s", cudaGetErrorString(e));
+  return DLM_OK;
+}
+
+template <bool BF16>
 int launch_typed(const VocabArgs& a, cudaStream_t stream) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int esz = BF16 ? 2 : 4;
-  const int64_t row_bytes = a.V * esz;
-  const int64_t want_ctas = 4LL * sms;  // resident CTAs at 4 per SM
-  // One CTA per row wherever there are rows enough to keep more than two CTAs
-  // per SM streaming: measured on this GPU (V = 151552, bf16), splitting rows
-  // over clusters wins only up to about 2 rows per SM (64 rows: 16 us against
-  // 21; 304: 22.6 against 24.9), and loses beyond (512 rows: 49.6 against 31.3,
-  // as each CTA's short chunks pay the memory latency once per row).
-  if (row_bytes < 65536 || a.N > 2LL * sms) {
-    const int64_t grid = a.N < 64LL * want_ctas ? a.N : 64LL * want_ctas;
-    if (VEC && a.N > want_ctas) {
-      // Several waves of rows: stage the loads through shared memory
-      // (measured at 32 x 512 x 151552: 0.692 ms against 0.722-0.733 for the
-      // register-loaded scan; with a single wave of rows the latter is as fast).
-      vocab_rows_kernel<BF16, VEC, true><<<static_cast<unsigned>(grid), kThreads, 0, stream>>>(a);
-    } else {
-      vocab_rows_kernel<BF16, VEC, false><<<static_cast<unsigned>(grid), kThreads, 0, stream>>>(a);
-    }
-  } else {
-    // Few long rows: split each over a cluster. Choose the cluster size that
-    // minimises the rows' share per CTA, ceil(N / clusters) / csize, with
-    // clusters = resident CTAs / csize (never more clusters than rows).
-    int csize = 2;
-    int64_t nclusters = 1;
-    double best = 1e30;
-    for (int c = 2; c <= 8; c *= 2) {
-      int64_t nc = want_ctas / c;
-      if (nc > a.N) nc = a.N;
-      const double cost = static_cast<double>((a.N + nc - 1) / nc) / c;
-      if (cost < best - 1e-9) {
-        best = cost;
-        csize = c;
-        nclusters = nc;
-      }
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = csize;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    // No more clusters than can be resident at once (one wave).
-    cfg.gridDim = dim3(static_cast<unsigned>(nclusters * csize));
-    int active = 0;
-    if (cudaOccupancyMaxActiveClusters(&active, vocab_cluster_kernel<BF16, VEC>, &cfg) == cudaSuccess && active > 0 &&
-        nclusters > active) {
-      nclusters = active;
-      cfg.gridDim = dim3(static_cast<unsigned>(nclusters * csize));
-    }
-    cudaGetLastError();  // an occupancy query that failed leaves the grid as computed
-    cudaError_t e = cudaLaunchKernelEx(&cfg, vocab_cluster_kernel<BF16, VEC>, a);
-    if (e != cudaSuccess)
-      return fail(DLM_ERR_CUDA, "vocab_confidence cluster launch: %s", cudaGetErrorString(e));
+  const int64_t row_bytes = a.V * (BF16 ? 2 : 4);
+  const int64_t resident = 4LL * sms;  // CTAs at 4 per SM
+  // Who works on a row (us measured on this GPU, 152 SMs, bf16, from a CUDA graph):
+  // * long rows, at most one per SM: a cluster, the larger the fewer rows there
+  //   are, up to about 2.6 CTAs per SM (V = 151552, clusters of 16 / 8 / 4: 1 row
+  //   3.4 / 3.8 / 4.9, 32 rows 5.4 / 4.8 / 5.4, 64 rows 8.7 / 6.9 / 6.5, 128 rows
+  //   17 / 12 / 10.3, where a CTA per row takes 11.1; rows twice as long: 64 rows
+  //   11.0 / 8.8 / 11.1, so 4 CTAs per SM for those);
+  // * short rows, enough of them to fill the SMs with warps: a warp (V = 1000 x
+  //   16384 rows 12.2 against 34 with a CTA per row, V = 4000 x 16384 27.9 against
+  //   48, V = 8000 x 8192 26.1 against 33.9, V = 16000 x 4096 23.7 against 27.3;
+  //   V = 32001 x 3000 36.2 against 34.4, and V = 4000 x 1000 the same either way);
+  // * else a CTA, its loads staged through shared memory (200 rows 15.4, from
+  //   registers 19.9, clusters of 4 15.7; 256 rows 15.7 / 20.6 / 17.5; 400 rows 21.8 /
+  //   23.8; 16384 rows 681 / 722) except where one wave of CTAs fills all places
+  //   (512 rows: 30.5 staged, 27.7 from registers).
+  if (row_bytes >= 65536 && a.N <= sms) {
+    const int64_t ctas = row_bytes > 400000 ? resident : 2 * resident / 3;
+    return launch_cluster<BF16>(a, a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4, stream);
   }
-  cudaError_t e = cudaGetLastError();
+  if (a.N > resident && (row_bytes <= 8192 || (row_bytes <= 40000 && a.N >= 24LL * sms))) {
+    const int64_t want = (a.N + kWarps - 1) / kWarps;
+    vocab_short_rows_kernel<BF16><<<static_cast<unsigned>(want < 64 * resident ? want : 64 * resident), kThreads, 0, stream>>>(a);
+  } else {
+    const unsigned grid = static_cast<unsigned>(a.N < 64 * resident ? a.N : 64 * resident);
+    if (a.N > 3LL * sms && a.N <= resident) vocab_rows_kernel<BF16, false><<<grid, kThreads, 0, stream>>>(a);
+    else vocab_rows_kernel<BF16, true><<<grid, kThreads, 0, stream>>>(a);
+  }
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
@@ -426,10 +463,7 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
 
 int launch_vocab_confidence(const VocabArgs& a, cudaStream_t stream) {
   if (a.N == 0) return DLM_OK;
-  const int esz = a.is_bf16 ? 2 : 4;
-  const bool vec = (reinterpret_cast<uintptr_t>(a.logits) % 16 == 0) && ((a.row_stride * esz) % 16 == 0);
-  if (a.is_bf16) return vec ? launch_typed<true, true>(a, stream) : launch_typed<true, false>(a, stream);
-  return vec ? launch_typed<false, true>(a, stream) : launch_typed<false, false>(a, stream);
+  return a.is_bf16 ? launch_typed<true>(a, stream) : launch_typed<false>(a, stream);
 }
 
 int launch_token_prob(const VocabArgs& a, const int32_t* tokens, const float* lse, float* prob,

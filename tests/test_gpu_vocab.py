@@ -174,3 +174,22 @@ def host_rows_planted(w, rows, pos, peak):
     x = host_logit_rows(w, 0, rows)
     x[:, pos] = np.float32(peak)
     return x
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N,V", [(3, 1), (5, 3), (4, 17), (9, 65537), (40, 4099), (700, 5), (700, 33), (1300, 4097),
+                                 (650, 9001)])
+def test_rows_off_16_byte_boundaries(dtype, N, V):
+    """Rows packed under an odd V, seen from every starting element: a cluster,
+    a CTA and a warp per row, rows shorter than one vector; equal maxima before,
+    inside and after a row's whole vectors, and -inf there."""
+    for off in range(8 if dtype == "bf16" else 4):
+        x = planted(N, V, N + V + off)
+        x[0, [0, V // 2, V - 1]] = 40.0
+        x[1, [V - 1, V // 2]] = 40.0
+        x[2, :] = -np.inf
+        x[2, V - 1 - off % V] = -3.0
+        flat = to_dev(np.concatenate([np.full(off, 99.0, np.float32), x.reshape(-1)]), dtype)
+        t = flat[off:].view(N, V)
+        ref = oracle.vocab_confidence(t.float().cpu().numpy())
+        check_vocab(*gpu_vocab(t), *ref, where=f"{dtype} {N}x{V} off {off}")
