@@ -10,7 +10,8 @@
 // Persistent CTAs (one per SM) walk work items = (vocabulary split, block of
 // 128 rows); items are ordered split-major, so the CTAs running at the same
 // time read the same weight tiles and those stay in L2. Per 128 x 256 output
-// tile:
+// tile (128 x 128 or 128 x 64 where the vocabulary is too small for a tile of
+// 256 columns on every SM):
 //   warp 0     TMA producer: hidden box 128 x 64 and weight box 256 x 64 per
 //              64-wide K step, through a 4-stage ring (48 KB a stage)
 //   warp 1     tensor-memory allocator and MMA issuer (all lanes run the loop,
@@ -48,17 +49,18 @@ namespace dlm {
 namespace {
 
 constexpr int kBM = 128;          // rows per tile = TMEM lanes
-constexpr int kBN = 256;          // vocabulary columns per tile
 constexpr int kBK = 64;           // K per stage: one 128-byte swizzle atom of bf16
-constexpr int kStages = 4;
 constexpr int kThreads = 256;     // warp 0 TMA, warp 1 MMA, warps 4-7 epilogue
 constexpr int kEpiWarp0 = 4;
-constexpr uint32_t kTmemCols = 512;
 constexpr int kABytes = kBM * kBK * 2;  // 16 KB (a stage of it holds LmParams::a_rows rows)
-constexpr int kBBytes = kBN * kBK * 2;  // 32 KB
 constexpr float kLog2e = 1.4426950408889634f;
 
+// kBN: vocabulary columns per tile, 256, or 128 or 64 where the vocabulary has
+// too few columns for a tile of 256 on every SM.
+template <int kBN>
 struct Smem {
+  static constexpr int kStages = kBN == 256 ? 4 : kBN == 128 ? 6 : 8;  // 192 KB
+  static constexpr int kBBytes = kBN * kBK * 2;
   alignas(1024) uint8_t a[kStages][kABytes];
   alignas(1024) uint8_t b[kStages][kBBytes];
   uint64_t full[kStages];     // stage loaded             (TMA -> MMA)
@@ -119,10 +121,13 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
   return __all_sync(0xffffffffu, ok);
 }
 
+template <int kBN>
 __global__ void __launch_bounds__(kThreads, 1)
     lmhead_kernel(const __grid_constant__ CUtensorMap th, const __grid_constant__ CUtensorMap tw, const LmParams p) {
   extern __shared__ uint8_t smem_raw[];
-  Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  constexpr int kStages = Smem<kBN>::kStages, kBBytes = Smem<kBN>::kBBytes;
+  constexpr uint32_t kTmemCols = 2 * kBN;  // two accumulators
+  Smem<kBN>& sm = *reinterpret_cast<Smem<kBN>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int kblocks = p.d / kBK;
@@ -416,43 +421,53 @@ int make_map_2d(CUtensorMap* map, const void* base, int64_t rows, int d, int64_t
 namespace {
 
 struct Split {
-  int csize, parts;  // CTAs per cluster, parts per row
+  int bn, csize, parts;  // columns per tile, CTAs per cluster, parts per row
 };
 
-// The split that leaves the busiest CTA the fewest 256-column tiles, plus a
-// small cost per item (pipeline fill, flush). Clusters (csize > 1) run one
-// item each, all at once. Measured for 64 rows x 151552 x 2048 (reading the
+template <int kBN>
+constexpr size_t smem_bytes() {
+  return sizeof(Smem<kBN>) + 1024;
+}
+
+template <int kBN>
+cudaError_t allow_smem() {
+  return cudaFuncSetAttribute(lmhead_kernel<kBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(smem_bytes<kBN>()));
+}
+
+// The split that leaves the busiest CTA the fewest columns (in tiles of 256;
+// narrower tiles read the hidden rows more often: 12 % more a halving), plus a
+// small cost per item (pipeline fill, flush). Narrow tiles win where 256 columns
+// leave SMs without one: 16 rows x 1000 x 4096 24.3 -> 19.4 us, x 512 9.7 -> 7.5, 100 x
+// 10000 x 2048 20.6 -> 16.7, 300 x 16000 x 2048 31.6 -> 30.2. Clusters (csize > 1) run
+// one item each, all at once. Measured for 64 rows x 151552 x 2048 (reading the
 // weight at the HBM copy rate: 93 us): 64 single CTAs 127 us, 64 clusters of 2
 // 101 us, 50 of 3 101 us, 32 of 4 101 us; 37 of 4, which are not all resident at
 // once, 141 us. 200 rows: 154 us with single CTAs, 117 us. From three row
 // blocks on, single CTAs fill the SMs.
-Split choose_split(int64_t row_blocks, int64_t vtiles, int sms, size_t smem) {
-  Split best{1, 1};
-  double best_cost = 1e300;
+template <int kBN>
+void choose_split(int64_t row_blocks, int64_t V, int sms, Split* best, double* best_cost) {
+  const int64_t vtiles = (V + kBN - 1) / kBN;
   for (int c = 1; c <= 4; c *= 2) {
     if (c > 1 && row_blocks * kLmMaxSplits >= sms) break;  // single CTAs already fill the SMs
-    const int64_t active = c == 1 ? sms : active_clusters(reinterpret_cast<const void*>(lmhead_kernel), c, kThreads, smem);
+    const int64_t active =
+        c == 1 ? sms : active_clusters(reinterpret_cast<const void*>(lmhead_kernel<kBN>), c, kThreads, smem_bytes<kBN>());
     for (int s = 1; s <= kLmMaxSplits && s <= (vtiles + c - 1) / c; ++s) {  // a cluster's last CTAs may have no tile
       const int64_t items = row_blocks * s;
       if (c > 1 && items > active) break;
       const int64_t rounds = (items + active - 1) / active;
-      const double cost = static_cast<double>(rounds) * (static_cast<double>((vtiles + s * c - 1) / (s * c)) + 0.5);
-      if (cost < best_cost - 1e-9) {
-        best_cost = cost;
-        best = {c, s};
+      const double tile = kBN / 256.0 * (0.88 + 0.12 * 256 / kBN);
+      const double cost = static_cast<double>(rounds) * (static_cast<double>((vtiles + s * c - 1) / (s * c)) * tile + 0.5);
+      if (cost < *best_cost - 1e-9) {
+        *best_cost = cost;
+        *best = {kBN, c, s};
       }
     }
   }
-  return best;
 }
 
-}  // namespace
-
-int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
-  if (a.N == 0) return DLM_OK;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+template <int kBN>
+int launch_tiles(const LmArgs& a, const Split& sp, int sms, cudaStream_t stream) {
   LmParams p;
   p.N = static_cast<int>(a.N);
   p.V = static_cast<int>(a.V);
@@ -460,11 +475,6 @@ int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
   p.row_blocks = static_cast<int>((a.N + kBM - 1) / kBM);
   p.vtiles = static_cast<int>((a.V + kBN - 1) / kBN);
   p.a_rows = a.N < kBM ? static_cast<int>((a.N + 7) / 8 * 8) : kBM;
-  const size_t smem = sizeof(Smem) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(lmhead_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead smem attribute: %s", cudaGetErrorString(e));
-  Split sp = choose_split(p.row_blocks, p.vtiles, sms, smem);
   p.csize = sp.csize;
   p.splits = sp.parts * sp.csize;
   p.items = p.row_blocks * sp.parts;
@@ -481,14 +491,15 @@ int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(sp.csize > 1 ? p.items * sp.csize : (p.items < sms ? p.items : sms)));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = smem_bytes<kBN>();
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim = {static_cast<unsigned>(sp.csize), 1, 1};
   cfg.attrs = attr;
   cfg.numAttrs = sp.csize > 1 ? 1 : 0;
-  if ((e = cudaLaunchKernelEx(&cfg, lmhead_kernel, mh, mw, p)) != cudaSuccess)
+  cudaError_t e = cudaLaunchKernelEx(&cfg, lmhead_kernel<kBN>, mh, mw, p);
+  if (e != cudaSuccess)
     return fail(DLM_ERR_CUDA, "lmhead launch: %s", cudaGetErrorString(e));
   const unsigned combine_grid = static_cast<unsigned>((a.N * 32 + kCombineThreads - 1) / kCombineThreads);
   lmhead_combine_kernel<<<combine_grid, kCombineThreads, 0, stream>>>(p.part_m, p.part_idx, p.part_s, p.N, sp.parts,
@@ -496,6 +507,28 @@ int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead combine launch: %s", cudaGetErrorString(e));
   return DLM_OK;
+}
+
+}  // namespace
+
+int launch_lmhead(const LmArgs& a, cudaStream_t stream) {
+  if (a.N == 0) return DLM_OK;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t row_blocks = (a.N + kBM - 1) / kBM;
+  cudaError_t e = allow_smem<256>();
+  if (e == cudaSuccess) e = allow_smem<128>();
+  if (e == cudaSuccess) e = allow_smem<64>();
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead smem attribute: %s", cudaGetErrorString(e));
+  Split sp{256, 1, 1};
+  double cost = 1e300;
+  choose_split<256>(row_blocks, a.V, sms, &sp, &cost);
+  choose_split<128>(row_blocks, a.V, sms, &sp, &cost);
+  choose_split<64>(row_blocks, a.V, sms, &sp, &cost);
+  if (sp.bn == 256) return launch_tiles<256>(a, sp, sms, stream);
+  if (sp.bn == 128) return launch_tiles<128>(a, sp, sms, stream);
+  return launch_tiles<64>(a, sp, sms, stream);
 }
 
 }  // namespace dlm

@@ -139,3 +139,18 @@ def test_few_row_blocks_split_over_clusters(N, V):
     check(gpu, hb.float().numpy(), wb.float().numpy(), f"N={N} V={V}")
     ref_am = oracle.lm_head_confidence(hb.float().numpy(), wb.float().numpy())[0]
     np.testing.assert_array_equal(gpu[0], ref_am)
+
+
+@pytest.mark.parametrize("N,V,d", [(5, 63, 4096), (64, 1000, 1024), (130, 129, 512), (70, 9000, 256), (300, 5000, 192),
+                                   (128, 18000, 64)])
+def test_narrow_tiles(N, V, d):
+    """Vocabularies too small for a 256-column tile on every SM: tiles of 128 and
+    64 columns, ragged last tiles, several row blocks; equal maxima in
+    neighbouring tiles."""
+    hb, wb = make_inputs(N, V, d, seed=N + V, peak_frac=0.5, peak=10.0)
+    am = oracle.lm_head_confidence(hb.float().numpy(), wb.float().numpy())[0].astype(np.int64)
+    wb[torch.from_numpy((am + 64) % V)] = wb[torch.from_numpy(am)]
+    gpu = gpu_lmhead(hb.to(dev()), wb.to(dev()))
+    check(gpu, hb.float().numpy(), wb.float().numpy(), f"N={N} V={V} d={d}")
+    ref_am = oracle.lm_head_confidence(hb.float().numpy(), wb.float().numpy())[0]
+    np.testing.assert_array_equal(gpu[0], ref_am)
