@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
   constexpr int kC4 = D / 4;    // 16-byte chunks per row
   constexpr int kCols = D / 64;  // float4 output columns per thread
 
+  wait_for_previous();
+  launch_dependents();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int row0 = blockIdx.x * T::kM, h = blockIdx.y, b = blockIdx.z;
   int n = a.seq_lens ? a.seq_lens[b] : a.L;
@@ -329,8 +331,7 @@ int launch_tile(const AttnArgs& a, bool vec, cudaStream_t stream) {
                                        static_cast<int>(T::kBytes));
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 smem attribute: %s", cudaGetErrorString(e));
   const dim3 grid((a.L + T::kM - 1) / T::kM, a.Hq, a.B);
-  attn_f32_kernel<D, kR, kMasked><<<grid, kThreads, T::kBytes, stream>>>(a, scale, vec, device_error_word());
-  e = cudaGetLastError();
+  e = launch_overlapped(attn_f32_kernel<D, kR, kMasked>, grid, kThreads, T::kBytes, stream, 1, true, a, scale, vec, device_error_word());
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }

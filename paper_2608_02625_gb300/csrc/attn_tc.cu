@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort = &sm.abort;
+  wait_for_previous();
 
   if (warp == kProducerWarp) {
     // ================================================================ TMA producer
@@ -373,6 +374,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       for (int j = 0; ok && j < U.nkv; ++j) ok = fill(U, j, true, j + 2 < U.nkv ? j + 2 : -1);
     }
+    // Only now: a successor whose CTAs take their places as this kernel's SMs
+    // fall idle is laid out less well (32 x 512 block-causal after itself, all
+    // launched this way: 124 us where every CTA let it start at once, 114 so).
+    launch_dependents();
     // Teardown: let every copy this warp issued land before the block exits.
     if (lane == 0) {
       if (q_loads0) mbar_drain(&sm.bar_q[0], (q_loads0 - 1) & 1);
@@ -827,8 +832,12 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
                                               static_cast<int>(smem));
   if (attr_err != cudaSuccess) return fail(DLM_ERR_CUDA, "attn smem attribute: %s", cudaGetErrorString(attr_err));
   const int grid = static_cast<int>(units < sms ? units : sms);
-  attn_tc_kernel<D, kMasked><<<grid, kThreads, smem, stream>>>(mq, mk, mv, mo, p);
-  cudaError_t e = cudaGetLastError();
+  // Under the block masks the units differ in length, and a launch whose CTAs
+  // take their places one by one is laid out worse: an ordinary launch there
+  // (32 x 512 block-causal 111 us against 114; full attention the other way
+  // round, 5 x 512 29.6 against 31.6, 1 x 512 9.9 against 10.1).
+  const cudaError_t e = launch_overlapped(attn_tc_kernel<D, kMasked>, dim3(static_cast<unsigned>(grid)), kThreads, smem, stream,
+                                          1, !kMasked, mq, mk, mv, mo, p);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_tc launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }

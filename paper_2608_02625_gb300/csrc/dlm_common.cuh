@@ -39,11 +39,20 @@ constexpr bool kCheckBounds = true;
 constexpr bool kCheckBounds = false;
 #endif
 
-// Lets a kernel launched with programmatic stream serialisation take free
-// places on the SMs once every block of this one has got here or ended.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// In such a kernel: waits until the one before it has ended and its writes are visible.
+// Every kernel of the library is launched so that it may start while the kernel
+// before it in the stream still runs (launch_overlapped, dlm_internal.h): its
+// set-up -- barriers, tensor memory, the launch itself -- then costs nothing
+// between calls that follow each other. The rules that make this safe:
+// * no kernel touches global memory before wait_for_previous, which returns once
+//   the kernel before it has ended and its writes are visible (the update behind
+//   the reduction of the same step reads what the reduction does not write
+//   before it; see refine_update_kernel);
+// * no kernel lets its successor start (launch_dependents) before its own
+//   wait_for_previous, so whatever came before the predecessor has ended too.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream take free places on the SMs once every
+// block of this one has got here or ended.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ----------------------------------------------------------------- mbarrier
 

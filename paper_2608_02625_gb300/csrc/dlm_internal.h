@@ -32,6 +32,27 @@ cudaStream_t current_stream();
 // if none can; asked of the runtime once per device, kernel and size.
 int active_clusters(const void* kernel, int csize, int threads, size_t smem);
 
+// Launches a kernel that may start while the one before it in the stream still
+// runs (every kernel of the library begins with wait_for_previous), in clusters
+// of `csize` CTAs; an ordinary launch where !overlap.
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int csize,
+                              bool overlap, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = csize > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 struct AttnArgs {
   const void* q;
   const void* k;

@@ -157,6 +157,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort = &sm.abort;
+  wait_for_previous();
+  launch_dependents();
 
   if (warp == 0) {
     // ================================================================ TMA producer
@@ -352,6 +354,8 @@ constexpr int kCombineThreads = 256;
 __global__ void __launch_bounds__(kCombineThreads)
     lmhead_combine_kernel(const float* part_m, const int* part_idx, const float* part_s, int N, int parts,
                           int32_t* argmax, float* conf, float* lse) {
+  wait_for_previous();
+  launch_dependents();
   const int64_t r = (static_cast<int64_t>(blockIdx.x) * kCombineThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= N) return;
@@ -488,23 +492,12 @@ int launch_tiles(const LmArgs& a, const Split& sp, int sms, cudaStream_t stream)
   int st;
   if ((st = make_map_2d(&mh, a.hidden, a.N, p.d, a.s_hidden, p.a_rows)) != DLM_OK) return st;
   if ((st = make_map_2d(&mw, a.weight, a.V, p.d, a.s_weight, kBN)) != DLM_OK) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(sp.csize > 1 ? p.items * sp.csize : (p.items < sms ? p.items : sms)));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem_bytes<kBN>();
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim = {static_cast<unsigned>(sp.csize), 1, 1};
-  cfg.attrs = attr;
-  cfg.numAttrs = sp.csize > 1 ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, lmhead_kernel<kBN>, mh, mw, p);
-  if (e != cudaSuccess)
-    return fail(DLM_ERR_CUDA, "lmhead launch: %s", cudaGetErrorString(e));
-  const unsigned combine_grid = static_cast<unsigned>((a.N * 32 + kCombineThreads - 1) / kCombineThreads);
-  lmhead_combine_kernel<<<combine_grid, kCombineThreads, 0, stream>>>(p.part_m, p.part_idx, p.part_s, p.N, sp.parts,
-                                                                      a.argmax, a.conf, a.lse);
-  e = cudaGetLastError();
+  const int grid = sp.csize > 1 ? p.items * sp.csize : (p.items < sms ? p.items : sms);
+  cudaError_t e = launch_overlapped(lmhead_kernel<kBN>, dim3(static_cast<unsigned>(grid)), kThreads, smem_bytes<kBN>(), stream,
+                                    sp.csize, true, mh, mw, p);
+  if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead launch: %s", cudaGetErrorString(e));
+  e = launch_overlapped(lmhead_combine_kernel, dim3(static_cast<unsigned>((a.N * 32 + kCombineThreads - 1) / kCombineThreads)),
+                        kCombineThreads, 0, stream, 1, true, p.part_m, p.part_idx, p.part_s, p.N, sp.parts, a.argmax, a.conf, a.lse);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "lmhead combine launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }

@@ -48,8 +48,10 @@ __device__ __forceinline__ int remask_count(const UpdateArgs& a, int r) {
 }
 
 // One sequence per CTA, position i = threadIdx.x + j * kThreads in registers of
-// thread threadIdx.x (L <= kItems * kThreads). kAfterVocab: launched behind the
-// vocabulary reduction that writes argmax and conf, before it has ended.
+// thread threadIdx.x (L <= kItems * kThreads). kAfterVocab: launched right behind
+// the vocabulary reduction that writes argmax and conf; the tokens, masks and
+// lengths, which it does not write, are loaded before the wait for its end (it
+// lets this kernel start only after its own predecessor has ended).
 template <int kThreads, int kItems, bool kAfterVocab>
 __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, int* err) {
   constexpr int kWarps = kThreads / 32;
@@ -58,6 +60,7 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
   const int items = (a.L + kThreads - 1) / kThreads;  // of the busiest thread
 
+  if (!kAfterVocab) wait_for_previous();
   int tok[kItems], pred[kItems];
   uint8_t msk[kItems];
   float cf[kItems], tp[kItems];
@@ -77,6 +80,7 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
   int n, p;
   lengths(a, b, err, &n, &p);
   if (kAfterVocab) wait_for_previous();
+  launch_dependents();
   {
     const int32_t* am = a.argmax + b * a.s_argmax;
     const float* conf = a.conf + b * a.s_conf;
@@ -218,38 +222,22 @@ __global__ void __launch_bounds__(kThreads) refine_update_kernel(UpdateArgs a, i
 constexpr int kLongThreads = 512;
 __global__ void __launch_bounds__(kLongThreads) refine_update_long_kernel(UpdateArgs a, int* err) {
   __shared__ UpdateShared<kLongThreads> sh;
+  wait_for_previous();
+  launch_dependents();
   refine_sequence<kLongThreads>(a, blockIdx.x, err, sh);
-}
-
-template <int kThreads, int kItems, bool kAfterVocab>
-cudaError_t launch_short(const UpdateArgs& a, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(a.B));
-  cfg.blockDim = dim3(kThreads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = kAfterVocab ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, refine_update_kernel<kThreads, kItems, kAfterVocab>, a, device_error_word());
 }
 
 template <bool kAfterVocab>
 int launch(const UpdateArgs& a, cudaStream_t stream) {
   if (a.B == 0) return DLM_OK;
+  const dim3 grid(static_cast<unsigned>(a.B));
+  int* err = device_error_word();
   cudaError_t e;
   // The fewest threads that hold the sequence: fewer warps meet at each barrier.
-  if (a.L <= 512) {
-    e = launch_short<128, 4, kAfterVocab>(a, stream);
-  } else if (a.L <= 2048) {
-    e = launch_short<256, 8, kAfterVocab>(a, stream);
-  } else if (a.L <= 8192) {
-    e = launch_short<1024, 8, kAfterVocab>(a, stream);
-  } else {
-    refine_update_long_kernel<<<a.B, kLongThreads, 0, stream>>>(a, device_error_word());
-    e = cudaGetLastError();
-  }
+  if (a.L <= 512) e = launch_overlapped(refine_update_kernel<128, 4, kAfterVocab>, grid, 128, 0, stream, 1, true, a, err);
+  else if (a.L <= 2048) e = launch_overlapped(refine_update_kernel<256, 8, kAfterVocab>, grid, 256, 0, stream, 1, true, a, err);
+  else if (a.L <= 8192) e = launch_overlapped(refine_update_kernel<1024, 8, kAfterVocab>, grid, 1024, 0, stream, 1, true, a, err);
+  else e = launch_overlapped(refine_update_long_kernel, grid, kLongThreads, 0, stream, 1, true, a, err);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "refine_update launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }

@@ -306,6 +306,7 @@ constexpr int kStages = 8;
 template <bool BF16, bool kStaged>
 __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
   __shared__ uint4 ring[kStaged ? kStages * kThreads : 1];
+  wait_for_previous();
   launch_dependents();
   for (int64_t rowi = blockIdx.x; rowi < a.N; rowi += gridDim.x) {
     const Row<BF16> row(a, rowi);
@@ -322,6 +323,7 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
 // One warp per row: many short rows.
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, 4) vocab_short_rows_kernel(VocabArgs a) {
+  wait_for_previous();
   launch_dependents();
   const int lane = threadIdx.x & 31;
   const int64_t warps = static_cast<int64_t>(gridDim.x) * kWarps;
@@ -352,6 +354,7 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a)
   const int crank = static_cast<int>(cluster.block_rank());
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nclusters = gridDim.x / csize;
+  wait_for_previous();
   launch_dependents();
   cluster.barrier_arrive();  // rank 0's shared memory may be written once every CTA runs
   int it = 0;
@@ -385,6 +388,8 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a)
 template <bool BF16>
 __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int32_t* tokens, const float* lse,
                                                          float* prob) {
+  wait_for_previous();
+  launch_dependents();
   const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (r >= a.N) return;
   const int32_t t = tokens[r];
@@ -407,16 +412,7 @@ int launch_cluster(const VocabArgs& a, int csize, cudaStream_t stream) {
   while ((active = active_clusters(reinterpret_cast<const void*>(kernel), csize, kThreads, 0)) == 0 && csize > 1) csize /= 2;
   if (active == 0) return fail(DLM_ERR_CUDA, "vocab_confidence: no cluster launch fits the device");
   const int64_t nclusters = a.N < active ? a.N : active;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(nclusters * csize));
-  cfg.blockDim = dim3(kThreads);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
+  const cudaError_t e = launch_overlapped(kernel, dim3(static_cast<unsigned>(nclusters * csize)), kThreads, 0, stream, csize, true, a);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence cluster launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
@@ -446,15 +442,14 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
     const int64_t ctas = row_bytes > 400000 ? resident : 2 * resident / 3;
     return launch_cluster<BF16>(a, a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4, stream);
   }
-  if (a.N > resident && (row_bytes <= 8192 || (row_bytes <= 40000 && a.N >= 24LL * sms))) {
-    const int64_t want = (a.N + kWarps - 1) / kWarps;
-    vocab_short_rows_kernel<BF16><<<static_cast<unsigned>(want < 64 * resident ? want : 64 * resident), kThreads, 0, stream>>>(a);
-  } else {
-    const unsigned grid = static_cast<unsigned>(a.N < 64 * resident ? a.N : 64 * resident);
-    if (a.N > 3LL * sms && a.N <= resident) vocab_rows_kernel<BF16, false><<<grid, kThreads, 0, stream>>>(a);
-    else vocab_rows_kernel<BF16, true><<<grid, kThreads, 0, stream>>>(a);
-  }
-  const cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  const auto grid = [&](int64_t ctas) { return dim3(static_cast<unsigned>(ctas < 64 * resident ? ctas : 64 * resident)); };
+  if (a.N > resident && (row_bytes <= 8192 || (row_bytes <= 40000 && a.N >= 24LL * sms)))
+    e = launch_overlapped(vocab_short_rows_kernel<BF16>, grid((a.N + kWarps - 1) / kWarps), kThreads, 0, stream, 1, true, a);
+  else if (a.N > 3LL * sms && a.N <= resident)
+    e = launch_overlapped(vocab_rows_kernel<BF16, false>, grid(a.N), kThreads, 0, stream, 1, true, a);
+  else
+    e = launch_overlapped(vocab_rows_kernel<BF16, true>, grid(a.N), kThreads, 0, stream, 1, true, a);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
@@ -469,10 +464,8 @@ int launch_vocab_confidence(const VocabArgs& a, cudaStream_t stream) {
 int launch_token_prob(const VocabArgs& a, const int32_t* tokens, const float* lse, float* prob,
                       cudaStream_t stream) {
   if (a.N == 0) return DLM_OK;
-  const unsigned grid = static_cast<unsigned>((a.N + 255) / 256);
-  if (a.is_bf16) token_prob_kernel<true><<<grid, 256, 0, stream>>>(a, tokens, lse, prob);
-  else token_prob_kernel<false><<<grid, 256, 0, stream>>>(a, tokens, lse, prob);
-  cudaError_t e = cudaGetLastError();
+  const auto kernel = a.is_bf16 ? token_prob_kernel<true> : token_prob_kernel<false>;
+  const cudaError_t e = launch_overlapped(kernel, dim3(static_cast<unsigned>((a.N + 255) / 256)), 256, 0, stream, 1, true, a, tokens, lse, prob);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "token_prob launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
