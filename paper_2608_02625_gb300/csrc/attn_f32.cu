@@ -80,7 +80,6 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
   constexpr int kCols = D / 64;  // float4 output columns per thread
 
   wait_for_previous();
-  launch_dependents();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int row0 = blockIdx.x * T::kM, h = blockIdx.y, b = blockIdx.z;
   int n = a.seq_lens ? a.seq_lens[b] : a.L;

@@ -374,9 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       for (int j = 0; ok && j < U.nkv; ++j) ok = fill(U, j, true, j + 2 < U.nkv ? j + 2 : -1);
     }
-    // Only now: a successor whose CTAs take their places as this kernel's SMs
-    // fall idle is laid out less well (32 x 512 block-causal after itself, all
-    // launched this way: 124 us where every CTA let it start at once, 114 so).
+    // Not earlier: 32 x 512 block-causal after itself, all launched this way,
+    // took 124 us where every CTA let the next one start at once, 114 so.
     launch_dependents();
     // Teardown: let every copy this warp issued land before the block exits.
     if (lane == 0) {

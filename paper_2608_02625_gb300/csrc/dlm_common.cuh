@@ -49,6 +49,11 @@ constexpr bool kCheckBounds = false;
 //   before it; see refine_update_kernel);
 // * no kernel lets its successor start (launch_dependents) before its own
 //   wait_for_previous, so whatever came before the predecessor has ended too.
+// Kernels of more than a few CTAs let it start when their CTAs end (which needs
+// no call), not before: CTAs that take their places one by one, as a running
+// kernel's leave, are spread unevenly over the SMs (400 vocabulary rows after
+// 400 others: 30.8 us where each CTA let the next kernel start at once, 21.7 us
+// evenly spread).
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream take free places on the SMs once every
 // block of this one has got here or ended.

@@ -158,7 +158,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort = &sm.abort;
   wait_for_previous();
-  launch_dependents();
 
   if (warp == 0) {
     // ================================================================ TMA producer
@@ -355,7 +354,6 @@ __global__ void __launch_bounds__(kCombineThreads)
     lmhead_combine_kernel(const float* part_m, const int* part_idx, const float* part_s, int N, int parts,
                           int32_t* argmax, float* conf, float* lse) {
   wait_for_previous();
-  launch_dependents();
   const int64_t r = (static_cast<int64_t>(blockIdx.x) * kCombineThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (r >= N) return;

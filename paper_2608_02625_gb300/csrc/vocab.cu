@@ -307,7 +307,6 @@ template <bool BF16, bool kStaged>
 __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
   __shared__ uint4 ring[kStaged ? kStages * kThreads : 1];
   wait_for_previous();
-  launch_dependents();
   for (int64_t rowi = blockIdx.x; rowi < a.N; rowi += gridDim.x) {
     const Row<BF16> row(a, rowi);
     int e;
@@ -324,7 +323,6 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads, 4) vocab_short_rows_kernel(VocabArgs a) {
   wait_for_previous();
-  launch_dependents();
   const int lane = threadIdx.x & 31;
   const int64_t warps = static_cast<int64_t>(gridDim.x) * kWarps;
   for (int64_t rowi = static_cast<int64_t>(blockIdx.x) * kWarps + (threadIdx.x >> 5); rowi < a.N; rowi += warps) {
@@ -355,7 +353,6 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nclusters = gridDim.x / csize;
   wait_for_previous();
-  launch_dependents();
   cluster.barrier_arrive();  // rank 0's shared memory may be written once every CTA runs
   int it = 0;
   for (int64_t rowi = blockIdx.x / csize; rowi < a.N; rowi += nclusters, ++it) {
@@ -389,7 +386,6 @@ template <bool BF16>
 __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int32_t* tokens, const float* lse,
                                                          float* prob) {
   wait_for_previous();
-  launch_dependents();
   const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (r >= a.N) return;
   const int32_t t = tokens[r];
