@@ -5,22 +5,29 @@
 // inputs call for fp32 arithmetic throughout (TF32 tensor cores would not hold
 // a 1e-5 error bound), so both products run as fp32 FMAs on register tiles.
 //
-// One CTA of 256 threads (16 x 16) computes 16 * kR query rows of one head
-// against 64-key tiles staged in shared memory: thread (ty, tx) owns the rows
-// ty * kR .. + kR - 1 and, of the scores, the keys tx + 16 j; of the output,
-// the columns 4 tx + 64 c .. + 3. The scores accumulate even and odd head-dim
-// elements in the two halves of packed fp32 FMAs (operands read as they lie in
-// memory, 16 bytes a load); a row's scores belong to one half-warp, so its
-// maximum is four shuffles and the numerators pass to the second product
-// through a half-warp's own slice of shared memory without a block barrier.
-// K and V have one buffer each: V_t is copied (cp.async) behind the scores of
-// tile t, K_{t+1} behind its softmax and second product.
+// The query heads that share a key/value head form one list of rows, head
+// after head (valid rows only), cut into tiles of 16 * kR rows, so that a tile
+// may run from one head into the next and no head ends in a partial tile of its
+// own (3 x 300, 32 / 4 heads: 129 us with tiles per head, 121 so). One CTA of
+// 256 threads (16 x 16) computes a tile against 64-key tiles staged in shared
+// memory: thread (ty, tx) owns the rows ty * kR .. + kR - 1 and, of the scores,
+// the keys tx + 16 j; of the output, the columns 4 tx + 64 c .. + 3. The scores
+// accumulate even and odd head-dim elements in the two halves of packed fp32
+// FMAs (operands read as they lie in memory, 16 bytes a load); a row's scores
+// belong to one half-warp, so its maximum is four shuffles and the numerators
+// pass to the second product through a half-warp's own slice of shared memory
+// without a block barrier. K and V have one buffer each: V_0 is copied beside
+// K_0, V_t behind the scores of tile t, K_{t+1} behind its softmax and second
+// product. Of the last key tile only the scores and products of the 16-key
+// groups and 4-key groups that hold keys are computed (26 x 21 positions, 7 keys,
+// block-local, D = 64: 9.1 us with whole tiles, 7.5 so; 8.3 with a warp per row).
 //
 // Bound by the FMA pipe: 80 % busy on the SMs that have a CTA (1 x 512, 32 / 4
-// heads, D = 128: 128 tiles of 128 rows on 152 SMs, 102 us against 1022 us for a
-// warp per query row; 8 x 512: 0.70 ms = 49 TFLOP/s).
+// heads, D = 128: 148 tiles of 112 rows on 152 SMs, 92 us against 1022 us for a
+// warp per query row; 8 x 512: 0.71 ms = 49 TFLOP/s).
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "dlm_common.cuh"
 #include "dlm_internal.h"
@@ -36,7 +43,8 @@ struct F32Tile {
   static constexpr int kM = 16 * kR;               // query rows per CTA
   static constexpr int kKStride = D + 4;           // floats; 16 lanes' rows then hit distinct banks
   static constexpr int kQGroup = kR * D + 4;       // one row group; two groups of a warp hit distinct banks
-  static constexpr int kPGroup = kKeys * kR + 4;   // numerators of one row group, [key][row]
+  static constexpr int kPRows = kR == 7 ? 8 : kR;  // rows of a key's numerators, padded to 16 bytes
+  static constexpr int kPGroup = kKeys * kPRows + 4;  // numerators of one row group, [key][row]
   static constexpr int kQ = 16 * kQGroup, kK = kKeys * kKStride, kV = kKeys * D, kP = 16 * kPGroup;
   static constexpr size_t kBytes = sizeof(float) * (kQ + kK + kV + kP);
 };
@@ -60,6 +68,11 @@ __device__ __forceinline__ void copy4(float* dst, const float* src, bool valid, 
   }
 }
 
+__device__ __forceinline__ void store4(float* dst, float4 x, bool vec) {
+  if (vec) *reinterpret_cast<float4*>(dst) = x;
+  else dst[0] = x.x, dst[1] = x.y, dst[2] = x.z, dst[3] = x.w;
+}
+
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void copies_wait() {
@@ -68,56 +81,91 @@ __device__ __forceinline__ void copies_wait() {
 
 __device__ __forceinline__ bool not_finite(float x) { return (__float_as_uint(x) & 0x7F800000u) == 0x7F800000u; }
 
+// Whether the row tiles of sequences of `len` positions are cut per head.
+__host__ __device__ __forceinline__ bool tiles_per_head(const AttnArgs& a, int len) {
+  return a.mask_mode == DLM_ATTN_BLOCK_LOCAL && len > kKeys;
+}
+
 template <int D, int kR, bool kMasked>
-__global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float scale, bool vec, int* err) {
+__global__ void __launch_bounds__(kThreads, kR == 2 || (kR == 4 && D == 64) ? 2 : 1) attn_f32_kernel(AttnArgs a, float scale, bool vec, int* err) {
   using T = F32Tile<D, kR>;
   extern __shared__ float4 smem_f4[];
   float* const sq = reinterpret_cast<float*>(smem_f4);
   float* const sk = sq + T::kQ;
   float* const sv = sk + T::kK;
   float* const sp = sv + T::kV;
+  __shared__ int2 row_of[T::kM];
   constexpr int kC4 = D / 4;    // 16-byte chunks per row
   constexpr int kCols = D / 64;  // float4 output columns per thread
 
   wait_for_previous();
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int row0 = blockIdx.x * T::kM, h = blockIdx.y, b = blockIdx.z;
+  const int g = blockIdx.y, b = blockIdx.z;
+  const int G = a.Hq / a.Hkv;
   int n = a.seq_lens ? a.seq_lens[b] : a.L;
+  int p = kMasked && a.prompt_lens ? a.prompt_lens[b] : 0;
   if (n < 0 || n > a.L) {
     if (tid == 0) set_device_error(err, DLM_DEVERR_LENGTH);
     n = n < 0 ? 0 : a.L;
   }
-  int p = 0;
-  if (kMasked && a.prompt_lens) {
-    p = a.prompt_lens[b];
-    if (p < 0 || p > n) {
-      if (tid == 0 && row0 < n) set_device_error(err, DLM_DEVERR_LENGTH);
-      p = p < 0 ? 0 : n;
-    }
+  if (kMasked && (p < 0 || p > n)) {
+    if (tid == 0 && n > 0) set_device_error(err, DLM_DEVERR_LENGTH);
+    p = p < 0 ? 0 : n;
   }
-  const int g = (h * a.Hkv) / a.Hq;
-  const float* qb = static_cast<const float*>(a.q) + b * a.sq[0] + h * a.sq[2];
+  const float* qb = static_cast<const float*>(a.q) + b * a.sq[0];
   const float* kb = static_cast<const float*>(a.k) + b * a.sk[0] + g * a.sk[2];
   const float* vb = static_cast<const float*>(a.v) + b * a.sv[0] + g * a.sv[2];
+  float* const ob = static_cast<float*>(a.out) + b * a.so[0];
+
+  // The group's rows: head after head, each n rows, or n rounded up to whole
+  // tiles under the block-local mask (a tile that ran from one head into the
+  // next would visit the blocks at both ends; where all keys are one tile that
+  // does not matter).
+  const int per = kMasked && tiles_per_head(a, n) ? (n + T::kM - 1) / T::kM * T::kM : n;
+  const int rows = G * per, row0 = blockIdx.x * T::kM;  // below 2^31: checked by the launcher
+  // Padding rows of the group's heads are zeros: written by the CTAs without a
+  // tile, or where there are none by all of them when they are done.
+  const int used = (rows + T::kM - 1) / T::kM, first_idle = used < static_cast<int>(gridDim.x) ? used : 0;
+  auto write_padding = [&] {
+    if (static_cast<int>(blockIdx.x) < first_idle) return;
+    const int pad = a.L - n;
+    for (int64_t e = static_cast<int64_t>(blockIdx.x - first_idle) * kThreads + tid; e < static_cast<int64_t>(G) * pad * kC4;
+         e += static_cast<int64_t>(gridDim.x - first_idle) * kThreads) {
+      const int z = static_cast<int>(e / kC4), head = z / pad;
+      store4(ob + (g * G + head) * a.so[2] + (n + z - head * pad) * a.so[1] + e % kC4 * 4, make_float4(0.f, 0.f, 0.f, 0.f), vec);
+    }
+  };
+  if (row0 >= rows) {
+    write_padding();
+    return;
+  }
+  // Row r of the tile: head and position (-1 past the head's last row).
+  if (tid < T::kM) {
+    const int rr = row0 + tid, head = rr / per, pos = rr - head * per;
+    row_of[tid] = rr < rows && pos < n ? make_int2(g * G + head, pos) : make_int2(0, -1);
+  }
+  __syncthreads();
 
   // Key tiles the CTA's rows may use: tile t starts at key 64 * (t < ka ? t : t + gap).
-  int tiles = row0 < n ? (n + kKeys - 1) / kKeys : 0, ka = tiles, gap = 0;
-  const int r_last = min(row0 + T::kM, n) - 1;
-  KeyRanges first{n, n, n}, last{n, n, n};  // of the CTA's first and last valid row
-  if (kMasked && tiles > 0) {
-    first = key_ranges(a.mask_mode, a.block, row0, n, p);
+  int tiles = (n + kKeys - 1) / kKeys, ka = tiles, gap = 0;
+  KeyRanges first{n, n, n}, last{n, n, n};  // of the CTA's lowest and highest position
+  if (kMasked) {
+    const int end = min(row0 + T::kM, rows) - 1;
+    const bool one_head = row0 / per == end / per;
+    const int r_first = one_head ? row0 % per : 0, r_last = one_head ? min(end % per, n - 1) : n - 1;
+    first = key_ranges(a.mask_mode, a.block, r_first, n, p);
     last = key_ranges(a.mask_mode, a.block, r_last, n, p);
     if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL || r_last < p) {
       ka = tiles = (last.hi1 + kKeys - 1) / kKeys;
     } else {
       const int prompt_end = (p + kKeys - 1) / kKeys;
-      const int own = (row0 < p ? p : first.lo2) / kKeys, end = (last.hi2 + kKeys - 1) / kKeys;
+      const int own = (r_first < p ? p : first.lo2) / kKeys, own_end = (last.hi2 + kKeys - 1) / kKeys;
       if (own <= prompt_end) {
-        ka = tiles = max(prompt_end, end);
+        ka = tiles = max(prompt_end, own_end);
       } else {
         ka = prompt_end;
         gap = own - prompt_end;
-        tiles = prompt_end + end - own;
+        tiles = prompt_end + own_end - own;
       }
     }
   }
@@ -126,7 +174,7 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
   if (kMasked) {
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
-      const KeyRanges kr = key_ranges(a.mask_mode, a.block, min(row0 + ty * kR + r, max(n - 1, 0)), n, p);
+      const KeyRanges kr = key_ranges(a.mask_mode, a.block, max(row_of[ty * kR + r].y, 0), n, p);
       hi1[r] = kr.hi1;
       lo2[r] = kr.lo2;
       hi2[r] = kr.hi2;
@@ -153,22 +201,23 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
   };
   auto key_of = [&](int t) { return kKeys * (t < ka ? t : t + gap); };
 
-  if (tiles > 0) {
-    for (int i = tid; i < T::kM * kC4; i += kThreads) {
-      const int r = i / kC4, c = i % kC4;
-      const bool valid = row0 + r < n;
-      copy4(sq + (r / kR) * T::kQGroup + (r % kR) * D + 4 * c, qb + (valid ? (row0 + r) * a.sq[1] + 4 * c : 0), valid, vec);
-    }
-    load_keys(sk, T::kKStride, kb, a.sk[1], key_of(0));
-    copies_commit();
-    copies_wait<0>();
-    __syncthreads();
+  for (int i = tid; i < T::kM * kC4; i += kThreads) {
+    const int r = i / kC4, c = i % kC4;
+    const int2 at = row_of[r];
+    copy4(sq + (r / kR) * T::kQGroup + (r % kR) * D + 4 * c,
+          qb + (at.y >= 0 ? at.x * a.sq[2] + at.y * a.sq[1] + 4 * c : 0), at.y >= 0, vec);
   }
+  load_keys(sk, T::kKStride, kb, a.sk[1], key_of(0));
+  copies_commit();
+  load_keys(sv, D, vb, a.sv[1], key_of(0));
+  copies_commit();
+  copies_wait<1>();
+  __syncthreads();
   const float* const q_mine = sq + ty * T::kQGroup;
   float* const p_mine = sp + ty * T::kPGroup;
   for (int t = 0; t < tiles; ++t) {
     const int key0 = key_of(t);
-    load_keys(sv, D, vb, a.sv[1], key0);
+    if (t > 0) load_keys(sv, D, vb, a.sv[1], key0);
     copies_commit();
     // ---- scores of keys key0 + tx + 16 j
     float2 s2[kR][4];
@@ -176,21 +225,28 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
     for (int r = 0; r < kR; ++r)
 #pragma unroll
       for (int j = 0; j < 4; ++j) s2[r][j] = make_float2(0.f, 0.f);
+    // The first kGroups * 16 keys of the tile.
+    auto scores = [&](auto groups) {
+      constexpr int kGroups = decltype(groups)::value;
 #pragma unroll 4
-    for (int c = 0; c < kC4; ++c) {
-      float4 kf[4];
+      for (int c = 0; c < kC4; ++c) {
+        float4 kf[kGroups];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) kf[j] = *reinterpret_cast<const float4*>(sk + (tx + 16 * j) * T::kKStride + 4 * c);
+        for (int j = 0; j < kGroups; ++j) kf[j] = *reinterpret_cast<const float4*>(sk + (tx + 16 * j) * T::kKStride + 4 * c);
 #pragma unroll
-      for (int r = 0; r < kR; ++r) {
-        const float4 qf = *reinterpret_cast<const float4*>(q_mine + r * D + 4 * c);
+        for (int r = 0; r < kR; ++r) {
+          const float4 qf = *reinterpret_cast<const float4*>(q_mine + r * D + 4 * c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          s2[r][j] = ffma2(make_float2(qf.x, qf.y), make_float2(kf[j].x, kf[j].y), s2[r][j]);
-          s2[r][j] = ffma2(make_float2(qf.z, qf.w), make_float2(kf[j].z, kf[j].w), s2[r][j]);
+          for (int j = 0; j < kGroups; ++j) {
+            s2[r][j] = ffma2(make_float2(qf.x, qf.y), make_float2(kf[j].x, kf[j].y), s2[r][j]);
+            s2[r][j] = ffma2(make_float2(qf.z, qf.w), make_float2(kf[j].z, kf[j].w), s2[r][j]);
+          }
         }
       }
-    }
+    };
+    if (n - key0 > 32) scores(std::integral_constant<int, 4>());
+    else if (n - key0 > 16) scores(std::integral_constant<int, 2>());
+    else scores(std::integral_constant<int, 1>());
     __syncthreads();  // every warp is done with K_t
     if (t + 1 < tiles) load_keys(sk, T::kKStride, kb, a.sk[1], key_of(t + 1));
     copies_commit();
@@ -230,11 +286,12 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      float* dst = p_mine + (tx + 16 * j) * kR;
+      float* dst = p_mine + (tx + 16 * j) * T::kPRows;
       if constexpr (kR >= 4) {
 #pragma unroll
         for (int r = 0; r < kR; r += 4)
-          *reinterpret_cast<float4*>(dst + r) = make_float4(s2[r][j].x, s2[r + 1][j].x, s2[r + 2][j].x, s2[r + 3][j].x);
+          *reinterpret_cast<float4*>(dst + r) =
+              make_float4(s2[r][j].x, s2[r + 1][j].x, s2[r + 2][j].x, r + 3 < kR ? s2[r + 3 < kR ? r + 3 : 0][j].x : 0.f);
       } else {
         *reinterpret_cast<float2*>(dst) = make_float2(s2[0][j].x, s2[1][j].x);
       }
@@ -256,26 +313,31 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
     }
     // ---- output += numerators x V
     if (!guard) {
-#pragma unroll 4
-      for (int key = 0; key < kKeys; ++key) {
-        float pr[kR];
-        if constexpr (kR >= 4) {
+      const int kend = min(kKeys, n - key0);  // the numerators and values past it are zeros
+#pragma unroll 1
+      for (int k4 = 0; k4 < kend; k4 += 4) {
 #pragma unroll
-          for (int r = 0; r < kR; r += 4) {
-            const float4 x = *reinterpret_cast<const float4*>(p_mine + key * kR + r);
-            pr[r] = x.x, pr[r + 1] = x.y, pr[r + 2] = x.z, pr[r + 3] = x.w;
+        for (int key = k4; key < k4 + 4; ++key) {
+          float pr[kR];
+          if constexpr (kR >= 4) {
+#pragma unroll
+            for (int r = 0; r < kR; r += 4) {
+              const float4 x = *reinterpret_cast<const float4*>(p_mine + key * T::kPRows + r);
+              pr[r] = x.x, pr[r + 1] = x.y, pr[r + 2] = x.z;
+              if (r + 3 < kR) pr[r + 3 < kR ? r + 3 : 0] = x.w;
+            }
+          } else {
+            const float2 x = *reinterpret_cast<const float2*>(p_mine + key * T::kPRows);
+            pr[0] = x.x, pr[1] = x.y;
           }
-        } else {
-          const float2 x = *reinterpret_cast<const float2*>(p_mine + key * kR);
-          pr[0] = x.x, pr[1] = x.y;
-        }
 #pragma unroll
-        for (int c = 0; c < kCols; ++c) {
-          const float4 vf = *reinterpret_cast<const float4*>(sv + key * D + 64 * c + 4 * tx);
+          for (int c = 0; c < kCols; ++c) {
+            const float4 vf = *reinterpret_cast<const float4*>(sv + key * D + 64 * c + 4 * tx);
 #pragma unroll
-          for (int r = 0; r < kR; ++r) {
-            o[r][2 * c] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.x, vf.y), o[r][2 * c]);
-            o[r][2 * c + 1] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.z, vf.w), o[r][2 * c + 1]);
+            for (int r = 0; r < kR; ++r) {
+              o[r][2 * c] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.x, vf.y), o[r][2 * c]);
+              o[r][2 * c + 1] = ffma2(make_float2(pr[r], pr[r]), make_float2(vf.z, vf.w), o[r][2 * c + 1]);
+            }
           }
         }
       }
@@ -286,7 +348,7 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
 #pragma unroll
         for (int r = 0; r < kR; ++r) {
           if (!(kpos < hi1[kMasked ? r : 0] || (kpos >= lo2[kMasked ? r : 0] && kpos < hi2[kMasked ? r : 0]))) continue;
-          const float w = p_mine[key * kR + r];
+          const float w = p_mine[key * T::kPRows + r];
 #pragma unroll
           for (int c = 0; c < kCols; ++c) {
             const float4 vf = *reinterpret_cast<const float4*>(sv + key * D + 64 * c + 4 * tx);
@@ -302,24 +364,19 @@ __global__ void __launch_bounds__(kThreads) attn_f32_kernel(AttnArgs a, float sc
 
 #pragma unroll
   for (int r = 0; r < kR; ++r) {
-    const int i = row0 + ty * kR + r;
 #pragma unroll
     for (int off = 8; off > 0; off >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], off);
-    if (i >= a.L) continue;
-    float* dst = static_cast<float*>(a.out) + b * a.so[0] + i * a.so[1] + h * a.so[2] + 4 * tx;
-    const bool valid = i < n;
-    const float inv = valid ? 1.0f / l[r] : 0.f;
+    const int2 at = row_of[ty * kR + r];
+    if (at.y < 0) continue;
+    float* dst = ob + at.x * a.so[2] + at.y * a.so[1] + 4 * tx;
+    const float inv = 1.0f / l[r];
 #pragma unroll
     for (int c = 0; c < kCols; ++c) {
       const float2 lo = o[r][2 * c], hi = o[r][2 * c + 1];
-      const float4 x = valid ? make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv) : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (vec) {
-        *reinterpret_cast<float4*>(dst + 64 * c) = x;
-      } else {
-        dst[64 * c] = x.x, dst[64 * c + 1] = x.y, dst[64 * c + 2] = x.z, dst[64 * c + 3] = x.w;
-      }
+      store4(dst + 64 * c, make_float4(lo.x * inv, lo.y * inv, hi.x * inv, hi.y * inv), vec);
     }
   }
+  write_padding();
 }
 
 template <int D, int kR, bool kMasked>
@@ -329,7 +386,9 @@ int launch_tile(const AttnArgs& a, bool vec, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(attn_f32_kernel<D, kR, kMasked>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(T::kBytes));
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 smem attribute: %s", cudaGetErrorString(e));
-  const dim3 grid((a.L + T::kM - 1) / T::kM, a.Hq, a.B);
+  const int64_t G = a.Hq / a.Hkv;
+  const int64_t tiles = tiles_per_head(a, a.L) ? G * ((a.L + T::kM - 1) / T::kM) : (G * a.L + T::kM - 1) / T::kM;
+  const dim3 grid(static_cast<unsigned>(tiles), a.Hkv, a.B);
   e = launch_overlapped(attn_f32_kernel<D, kR, kMasked>, grid, kThreads, T::kBytes, stream, 1, true, a, scale, vec, device_error_word());
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_f32 launch: %s", cudaGetErrorString(e));
   return DLM_OK;
@@ -349,19 +408,28 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // Query rows per CTA (16 kR): the kR whose busiest SM is done first. In units
-  // of one 128-row CTA, a 64-row one takes 0.7 and a 32-row one 0.55 alone on
-  // an SM; a further one beside it adds 0.7 (0.54 with D = 64, where two fit)
-  // and 0.44. Measured at D = 128, 32 heads, per 64-key tile: 13.1 / 9.1 / 7.0 us
-  // alone, 11.5 us for two 32-row CTAs. L = 512: 104 / 136 / 175 us with 128 / 64 /
-  // 32 rows; L = 256: 53 / 36 / 46; L = 128: 28 / 20 / 15 (a warp per query row,
-  // the kernel before: 1022 us at L = 512).
-  const double heads = static_cast<double>(a.B) * a.Hq;
-  auto cost = [&](int rows, double alone, double more) {
-    return alone + (ceil(heads * ((a.L + rows - 1) / rows) / sms) - 1.0) * more;
+  // of one 128-row CTA, a 112-row one takes 0.94, a 64-row one 0.7 and a 32-row one
+  // 0.55 alone on an SM; a further one beside it adds as much, but 0.54 for 64 rows
+  // at D = 64, where two fit, and 0.44 for 32. Measured at D = 128, 32 heads, per
+  // 64-key tile: 13.1 / 9.1 / 7.0 us alone for 128 / 64 / 32 rows, 11.5 us for two
+  // 32-row CTAs; whole calls: L = 512 100 / 92 / 136 / 175 us with 128 / 112 / 64 / 32
+  // rows, L = 256 53 / - / 33 / 46, L = 128 28 / - / 20 / 14.
+  const int64_t G = a.Hq / a.Hkv;
+  if (G * (a.L + 128LL) > 0x7FFFFFFFLL) return fail(DLM_ERR_SHAPE, "too many query rows per key/value head");
+  auto tiles = [&](int m) {
+    return tiles_per_head(a, a.L) ? G * ((a.L + m - 1) / m) : (G * a.L + m - 1) / m;
   };
-  const double c8 = cost(128, 1.0, 1.0), c4 = cost(64, 0.7, D == 64 ? 0.54 : 0.7), c2 = cost(32, 0.55, 0.44);
-  if (c8 <= c4 && c8 <= c2) return launch_tile<D, 8, kMasked>(a, vec, stream);
-  if (c4 <= c2) return launch_tile<D, 4, kMasked>(a, vec, stream);
+  auto cost = [&](int m, double alone, double more) {
+    return alone + (ceil(static_cast<double>(tiles(m)) * a.B * a.Hkv / sms) - 1.0) * more;
+  };
+  // 112 rows only where they make more tiles (7 x 150, 8 heads each its own: the same
+  // 112 CTAs either way, 20.0 us with 128 rows and 23.8 with 112).
+  const double c8 = cost(128, 1.0, 1.0), c7 = tiles(112) > tiles(128) ? cost(112, 0.94, 0.94) : c8 + 1.0,
+               c4 = cost(64, 0.7, D == 64 ? 0.54 : 0.7), c2 = cost(32, 0.55, 0.44);
+  const double best = fmin(fmin(c8, c7), fmin(c4, c2));
+  if (c8 == best) return launch_tile<D, 8, kMasked>(a, vec, stream);
+  if (c7 == best) return launch_tile<D, 7, kMasked>(a, vec, stream);
+  if (c4 == best) return launch_tile<D, 4, kMasked>(a, vec, stream);
   return launch_tile<D, 2, kMasked>(a, vec, stream);
 }
 

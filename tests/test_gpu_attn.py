@@ -267,12 +267,15 @@ def test_workload_tiles_bit_identical():
     (3, 33, 2, 1, 128),      # 32-row tiles, the second nearly empty
     (1, 128, 16, 16, 64),    # whole 32-row tiles
     (9, 129, 8, 2, 64), (3, 129, 20, 4, 128),    # 64-row tiles, a last one of one row
-    (5, 257, 16, 4, 128), (20, 65, 32, 8, 64),   # 128-row tiles
+    (5, 257, 16, 4, 128), (2, 337, 24, 2, 64),   # 112-row tiles that run from head to head
+    (20, 65, 32, 8, 64), (2, 300, 152, 2, 128),  # 64- and 128-row ones
+    (7, 48, 40, 8, 64), (1, 15, 1, 1, 64),       # 128- and 32-row tiles with fewer keys than a key tile
 ])
 def test_f32_tile_edges(B, L, Hq, Hkv, D):
-    """Each query tile of the fp32 kernel (32, 64 and 128 rows, chosen by the
-    number of tiles), with lengths at the edges of the 64-key tiles."""
-    sl = [(L, L - 1, 1, 64, 65, 0, 63)[b % 7] for b in range(B)]
+    """Each query tile of the fp32 kernel (32, 64, 112 and 128 rows, chosen
+    by the number of tiles), with lengths at the edges of the 64-key tiles and of the
+    16-key groups of a last one."""
+    sl = [(L, L - 1, 1, 64, 65, 0, 63, 16, 17, 33)[b % 10] for b in range(B)]
     run_case(B, L, Hq, Hkv, D, [min(n, L) for n in sl], 1.0, "f32", seed=B + L)
 
 

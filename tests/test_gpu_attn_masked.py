@@ -137,10 +137,11 @@ def test_workload_full_size(mode):
 
 
 @pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
-@pytest.mark.parametrize("Hq", [2, 80, 152])
+@pytest.mark.parametrize("Hq", [2, 40, 80, 152])
 def test_f32_values_outside_a_mask_never_reach_a_row(mode, Hq):
     """A NaN or an infinity in v at a key reaches the rows that attend to the key
-    and no other, with each query tile of the fp32 kernel (32, 64, 128 rows)."""
+    and no other, with each query tile of the fp32 kernel (32, 64,
+    112, 128 rows)."""
     L, p, block, key = 128, 20, 40, 97   # blocks [20, 60), [60, 100), [100, 128)
     q, k, v = rand_qkv(1, L, Hq, 1, 64, 1.0, "f32", seed=Hq)
     bad = v.clone()
@@ -153,3 +154,18 @@ def test_f32_values_outside_a_mask_never_reach_a_row(mode, Hq):
         attends[100:] = True
     assert torch.equal(got[0, ~attends], good[0, ~attends])
     assert not torch.isfinite(got[0, attends]).any()
+
+
+@pytest.mark.parametrize("mode,block", [(CAUSAL, 64), (LOCAL, 64), (CAUSAL, 9), (LOCAL, 20)])
+@pytest.mark.parametrize("B,L,Hq,Hkv,D", [
+    (2, 337, 24, 2, 128),    # 112-row tiles from head to head, 128-row ones per head when local
+    (3, 225, 28, 4, 64),     # 64-row tiles
+    (9, 33, 12, 2, 64),      # 32-row tiles; a single key tile: from head to head in both modes
+])
+def test_f32_tiles_across_heads(B, L, Hq, Hkv, D, mode, block):
+    """Tiles whose rows belong to several heads, ragged lengths and prompts, with
+    padding rows written by CTAs without rows and by CTAs that have some."""
+    sl = [(L, 65, 17, 64, 0, 1, 16, 33, L - 1)[b % 9] for b in range(B)]
+    sl = [min(n, L) for n in sl]
+    pl = [(0, n // 3, n)[b % 3] for b, n in enumerate(sl)]
+    run(B, L, Hq, Hkv, D, sl, pl, mode, block, 1.0, "f32", seed=L + block + mode)
