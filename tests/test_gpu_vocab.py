@@ -193,3 +193,18 @@ def test_rows_off_16_byte_boundaries(dtype, N, V):
         t = flat[off:].view(N, V)
         ref = oracle.vocab_confidence(t.float().cpu().numpy())
         check_vocab(*gpu_vocab(t), *ref, where=f"{dtype} {N}x{V} off {off}")
+
+
+@pytest.mark.parametrize("dtype,peak", [("bf16", 77.5), ("f32", 77.3), ("f32", -301.7)])
+@pytest.mark.parametrize("N,V", [(2, 40001), (300, 9001), (700, 1000)])
+def test_large_maxima_cost_no_accuracy(dtype, peak, N, V):
+    """m log2(e) rounded is off by up to 2^-18 here (half an ulp of 435), the same
+    way for every term; the sum must not keep that. Left are the rounding of
+    ex2.approx (2^-22), of x - m from the FMA and of the sums (a few 2^-24)."""
+    rng = np.random.default_rng(V)
+    x = (peak - rng.integers(0, 9, (N, V)) / 2).astype(np.float32)
+    t = to_dev(x, dtype)
+    _, conf, lse = gpu_vocab(t)
+    y = t.double()
+    exact = torch.exp(y.max(1).values - torch.logsumexp(y, 1)).cpu().numpy()
+    assert np.abs(conf / exact - 1).max() <= 2.0 ** -20
