@@ -443,9 +443,22 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
   //   registers 19.9, clusters of 4 15.7; 256 rows 15.7 / 20.6 / 17.5; 400 rows 21.8 /
   //   23.8; 16384 rows 681 / 722) except where one wave of CTAs fills all places
   //   (512 rows: 30.5 staged, 27.7 from registers).
+  // Around one row per SM (clusters of 4, of 2, a CTA per row): where the clusters of 4 no
+  // longer all fit at once (152 rows 14.1 / 12.5 / 11.0, fp32 23.3 / 19.9 / 17.9) and, rows
+  // of 200 KB and less in bf16, a little before (V = 100000, 100 rows 6.2 / 7.7 / 7.3, 136
+  // rows 7.9 / 8.8 / 7.3; V = 40000, 136 rows 5.2 / 4.5 / 4.2, but fp32 5.6 / 6.5 / 5.5), a
+  // CTA per row; past one row per SM some SMs have two rows and most one, which halves
+  // of rows even out for long bf16 rows (160 rows 14.3 / 13.4 / 14.7, 200 rows 15.5 / 14.3 /
+  // 15.0, 230 rows 16.9 / 15.8 / 15.1; V = 64000, 160 rows 7.7 / 6.8 / 7.4; fp32 160 rows
+  // 23.6 / 20.3 / 19.2).
   if (row_bytes >= 65536 && a.N <= sms) {
     const int64_t ctas = row_bytes > 400000 ? resident : 2 * resident / 3;
-    return launch_cluster<BF16>(a, a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4, stream);
+    const int csize = a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4;
+    const int most = BF16 && row_bytes <= 200000 ? 3 * sms / 4
+                                                 : active_clusters(reinterpret_cast<const void*>(vocab_cluster_kernel<BF16>), 4, kThreads, 0);
+    if (csize > 4 || a.N <= most) return launch_cluster<BF16>(a, csize, stream);
+  } else if (BF16 && row_bytes >= 100000 && a.N > sms && 3 * a.N <= 4 * sms) {
+    return launch_cluster<BF16>(a, 2, stream);
   }
   cudaError_t e;
   const auto grid = [&](int64_t ctas) { return dim3(static_cast<unsigned>(ctas < 64 * resident ? ctas : 64 * resident)); };
