@@ -12,7 +12,7 @@
 // both. When even single tiles all fit on the SMs at once (a single short
 // sequence) a unit is one tile in slot 0 and slot 1 idles. The kernel
 // is persistent: one CTA per SM walks units blockIdx.x, blockIdx.x +
-// gridDim.x, ...; the next unit's query tiles load as soon as the slot's last
+// gridDim.x, ..., or takes them one by one (launch_d); the next unit's query tiles load as soon as the slot's last
 // score MMA has run, and its first score MMAs overlap the epilogue.
 //
 // Keys are processed in 64-key sub-tiles so that each slot's scores can be
@@ -20,7 +20,7 @@
 // softmax warps work on S(j), which keeps the serial chain
 // softmax -> PV -> next scores off the critical path.
 //
-// Warp roles (352 threads):
+// Warp roles (352 threads, 384 with warp 11):
 //   warps 0-3  softmax + epilogue of slot 0 (thread t owns query row t = TMEM lane t)
 //   warps 4-7  softmax + epilogue of slot 1
 //   warp 8     TMA producer: Q per unit and slot; then the unit's key/value
@@ -33,6 +33,8 @@
 //   warp 9     tensor-memory allocator; MMA issuer of slot 0 (one lane elected
 //              per instruction)
 //   warp 10    MMA issuer of slot 1
+//   warp 11    (long sequences, kTake) takes further units by cluster launch
+//              control
 // Tensor memory (512 columns x 128 lanes x 32 bit), slot i at column 256 i:
 //   S_i buffers 0 and 1   fp32 128 x 64 at +0 and +64 (sub-tile j uses buffer j % 2)
 //   P_i                    bf16 numerators over the first 32 columns of that buffer
@@ -72,9 +74,13 @@ namespace {
 constexpr int kTile = 128;          // query rows per tile
 constexpr int kSub = 64;            // keys per sub-tile
 constexpr int kRing = 4;            // K/V ring entries (two sub-tiles each)
-constexpr int kThreads = 352;
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp0 = 9;   // warps 9 and 10 issue the MMAs of slots 0 and 1
+constexpr int kTakeWarp = 11;  // kTake: takes the units of CTAs that have not started
+template <bool kTake>
+constexpr int kThreads = 32 * (kTake ? kTakeWarp + 1 : kTakeWarp);
+constexpr int kTakes = 2;      // answers kept: the loads may be that many units ahead of the softmax
+constexpr int kAskAhead = 3;   // key sub-tiles before the end of a unit's loads
 constexpr uint32_t kTmemCols = 512;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 
@@ -99,6 +105,10 @@ struct Smem {
   uint64_t bar_ofree[2];      // O_i read out by the epilogue         (epilogue -> MMA)
   uint64_t bar_vtmp;          // private fill of a partial V sub-tile
   uint64_t bar_done[2];       // every MMA of issuer i completed
+  alignas(16) uint8_t taken[kTakes][16];  // answer k names unit k + 1, in slot k % kTakes (kTake)
+  uint64_t bar_ask;           // near the end of the unit's loads      (TMA -> warp 11)
+  uint64_t bar_taken[kTakes];  // slot answered                       (launch control -> all)
+  uint64_t bar_read[kTakes];   // slot read by every other warp        (all -> warp 11)
   uint32_t tmem_base;
   int abort;
   int unit_flag;   // units whose first slot-0 hand-off happened
@@ -127,9 +137,11 @@ FastDiv make_fastdiv(int d) {
 }
 
 struct TcParams {
-  int B, L, Hq, Hkv, G, mtiles, units_per_bg, units;
+  int B, L, Hq, Hkv, G, mtiles, units_per_bg, units;  // units_per_bg: per head and level
   int tpu;  // query tiles per unit: 2 (both slots), 1 (slot 0 only: few tiles)
   FastDiv div_upb, div_hkv, div_g;  // by units_per_bg, Hkv, G
+  FastDiv div_level;  // by level_units (block masks)
+  int level_units, u_top;  // units of a level, a head's first unit of level 0
   int mask_mode, block;
   const int32_t* seq_lens;
   const int32_t* prompt_lens;
@@ -157,8 +169,12 @@ struct Unit {
 template <bool kMasked>
 __device__ __forceinline__ Unit decode_unit(const TcParams& p, int unit) {
   Unit U;
-  const int bg = p.div_upb.div(unit);
-  const int u = unit - bg * p.units_per_bg;
+  // Head after head (one level), or by row tile, the last first, the units of one
+  // row tile and key/value head side by side (a level per row tile).
+  const int level = kMasked ? p.div_level.div(unit) : 0;
+  const int in_level = kMasked ? unit - level * p.level_units : unit;
+  const int bg = p.div_upb.div(in_level);
+  const int u = in_level - bg * p.units_per_bg + (kMasked ? p.u_top - level * p.units_per_bg : 0);
   U.b = p.div_hkv.div(bg);
   U.g = bg - U.b * p.Hkv;
   int n = p.seq_lens ? p.seq_lens[U.b] : p.L;
@@ -240,9 +256,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // kMasked: the block masks of dlm_attn_masked (a separate instantiation, so
-// that full attention carries none of their per-row bookkeeping).
-template <int D, bool kMasked>
-__global__ void __launch_bounds__(kThreads, 1)
+// that full attention carries none of their per-row bookkeeping). kTake: one CTA
+// per unit is launched, and a running one takes those that have not started; else
+// a CTA's units are one grid apart.
+template <int D, bool kMasked, bool kTake>
+__global__ void __launch_bounds__(kThreads<kTake>, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
                    const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap to,
                    const TcParams p) {
@@ -275,6 +293,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&sm.bar_full[r], 1);
       mbar_init(&sm.bar_empty[r], 2);  // one release per slot
     }
+    mbar_init(&sm.bar_ask, 1);
+    for (int r = 0; r < kTakes; ++r) {
+      mbar_init(&sm.bar_taken[r], 1);
+      mbar_init(&sm.bar_read[r], kTakeWarp);  // warps 0 .. 10
+    }
     mbar_init(&sm.bar_vtmp, 1);
     mbar_init(&sm.bar_done[0], 1);
     mbar_init(&sm.bar_done[1], 1);
@@ -294,7 +317,39 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort = &sm.abort;
   wait_for_previous();
 
-  if (warp == kProducerWarp) {
+  // The unit after `unit`, -1 after the last (kTake: the one that warp 11 asked for).
+  uint32_t reads = 0;
+  auto next_unit = [&](int unit) -> int {
+    if constexpr (kTake) {
+      const uint32_t r = reads % kTakes;
+      if (!warp_wait(&sm.bar_taken[r], (reads / kTakes) & 1, abort, p.err, p.wait_ns)) return -1;
+      ++reads;
+      unit = taken_cta(sm.taken[r]);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.bar_read[r]);
+      return unit;
+    } else {
+      unit += gridDim.x;
+      return unit < p.units ? unit : -1;
+    }
+  };
+
+  if (kTake && warp == kTakeWarp) {
+    // ================================================================ further units
+    if (lane == 0) {
+      bool drop = false;  // a wait ran out: the units left are taken and not run
+      for (uint32_t k = 0;; ++k) {
+        const uint32_t r = k % kTakes;
+        if (!drop) drop = !mbar_wait_for(&sm.bar_ask, k & 1, abort, p.err, p.wait_ns);
+        if (!drop && k >= kTakes) drop = !mbar_wait_for(&sm.bar_read[r], (k / kTakes - 1) & 1, abort, p.err, p.wait_ns);
+        fence_proxy_async_smem();  // the slot was read before it is written again
+        mbar_arrive_expect_tx(&sm.bar_taken[r], sizeof(sm.taken[r]));
+        take_cta(sm.taken[r], &sm.bar_taken[r]);
+        if (!mbar_drain(&sm.bar_taken[r], (k / kTakes) & 1) || taken_cta(sm.taken[r]) < 0) break;
+      }
+    }
+    __syncwarp();
+  } else if (warp == kProducerWarp) {
     // ================================================================ TMA producer
     int q_loads0 = 0, q_loads1 = 0;  // query loads per slot (= bar_q / bar_qfree phases)
     int fills = 0;             // ring fills issued; slot fills % kRing, phase (fills / kRing) & 1
@@ -353,9 +408,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       ++fills;
       return true;
     };
-    for (int unit = blockIdx.x; ok && unit < p.units; unit += gridDim.x) {
+    for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
       const Unit U = decode_unit<kMasked>(p, unit);
-      if (U.nkv == 0) continue;
+      // Late, so that the CTAs ask in the order in which they end (2 x 2146
+      // block-causal 25 us; all asking at the start of their unit 39).
+      auto ask = [&] {
+        if (kTake && lane == 0) mbar_arrive(&sm.bar_ask);
+      };
+      const int ask_at = max(U.nkv - kAskAhead, 0);
+      if (U.nkv == 0) {
+        ask();
+        continue;
+      }
       // The unit's first key tiles need only ring slots: start them before
       // the query tiles, which wait for the previous unit's last score MMAs.
       ok = fill(U, 0, false, U.nkv >= 2 ? 1 : -1);
@@ -372,7 +436,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (i) ++q_loads1; else ++q_loads0;
       }
       if (!ok) break;
-      for (int j = 0; ok && j < U.nkv; ++j) ok = fill(U, j, true, j + 2 < U.nkv ? j + 2 : -1);
+      for (int j = 0; ok && j < U.nkv; ++j) {
+        if (j == ask_at) ask();
+        ok = fill(U, j, true, j + 2 < U.nkv ? j + 2 : -1);
+      }
     }
     // Not earlier: 32 x 512 block-causal after itself, all launched this way,
     // took 124 us where every CTA let the next one start at once, 114 so.
@@ -446,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       int p_seen = 0;     // bar_p hand-offs consumed
       int f = 0;          // ring fills consumed
       bool ok = true;
-      for (int unit = blockIdx.x; ok && unit < p.units; unit += gridDim.x) {
+      for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
         const Unit U = decode_unit<kMasked>(p, unit);
         if (U.nkv == 0) continue;
         const bool run = U.run[i];
@@ -524,7 +591,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int pvm_seen = 0;   // bar_pvm phases consumed
     int units_run = 0;  // bar_o phases consumed
     bool ok = true;
-    for (int unit = blockIdx.x; ok && unit < p.units; unit += gridDim.x) {
+    for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
       const Unit U = decode_unit<kMasked>(p, unit);
       const int f0 = f_next;
       if (U.nkv > 0) f_next += U.nkv + 1;
@@ -812,7 +879,6 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   const int forced = attn_tiles_per_unit();
   p.tpu = forced ? forced : (2 * pairs <= sms ? 1 : 2);
   p.units_per_bg = (p.G * p.mtiles + p.tpu - 1) / p.tpu;
-  p.div_upb = make_fastdiv(p.units_per_bg);
   p.div_hkv = make_fastdiv(p.Hkv);
   p.div_g = make_fastdiv(p.G);
   const long long units = static_cast<long long>(a.B) * a.Hkv * p.units_per_bg;
@@ -831,16 +897,41 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   p.err = device_error_word();
   p.wait_ns = wait_budget_ns();
   const size_t smem = sizeof(Smem<D>) + 1024;
-  cudaError_t attr_err = cudaFuncSetAttribute(attn_tc_kernel<D, kMasked>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              static_cast<int>(smem));
-  if (attr_err != cudaSuccess) return fail(DLM_ERR_CUDA, "attn smem attribute: %s", cudaGetErrorString(attr_err));
-  const int grid = static_cast<int>(units < sms ? units : sms);
+  // Units differ in length: by their sequence, by padding, under the block-causal
+  // mask by their row tile. Long sequences (12 row tiles): one CTA per unit is
+  // launched and whichever running CTA is free takes the next, instead of a fixed
+  // share per CTA (4 x 1836, n = 1241 .. 1633, 32 / 4 heads: 120 us against 151; 13 x 1685 (4 / 1
+  // heads) 46 / 64; 28 x 1914 (4 / 1, D = 64) 103 / 119; block-causal 2 x 2146 26 / 38, 35 x
+  // 1897 (4 / 1) 62 / 82; 5 x 2073, nearly all of one length, 168 / 166). On the whole GPU a
+  // unit is taken every 35 to 60 ns at best, which many short ones outrun (41 x
+  // 1664, n = 445 .. 455, 2132 units 76 / 71, block-causal 83 / 66; 32 x 512 block-causal
+  // 112 / 107), and where there are many rounds of them shares are nearly even
+  // anyway (8 x 2048 404 / 411): up to 10 rounds.
+  const long long rounds = (units + sms - 1) / sms;
+  const bool take = a.mask_mode != DLM_ATTN_BLOCK_LOCAL && p.mtiles >= 12 && units > sms && rounds <= 10;
+  const int tile_units = p.G % p.tpu == 0 ? p.G / p.tpu : 1;
+  p.level_units = p.units;
+  p.u_top = 0;
+  if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL && take) {
+    // By row tile, the last and so the longest units first.
+    p.u_top = p.units_per_bg - tile_units;
+    p.units_per_bg = tile_units;
+    p.level_units = tile_units * a.B * a.Hkv;
+  }
+  p.div_level = make_fastdiv(p.level_units);
+  p.div_upb = make_fastdiv(p.units_per_bg);
+  const int grid = static_cast<int>(take || units < sms ? units : sms);
   // Under the block masks the units differ in length, and a launch whose CTAs
   // take their places one by one is laid out worse: an ordinary launch there
   // (32 x 512 block-causal 111 us against 114; full attention the other way
   // round, 5 x 512 29.6 against 31.6, 1 x 512 9.9 against 10.1).
-  const cudaError_t e = launch_overlapped(attn_tc_kernel<D, kMasked>, dim3(static_cast<unsigned>(grid)), kThreads, smem, stream,
-                                          1, !kMasked, mq, mk, mv, mo, p);
+  const auto launch = [&](auto kernel, int threads) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    return e != cudaSuccess ? e : launch_overlapped(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, stream, 1, !kMasked,
+                                                    mq, mk, mv, mo, p);
+  };
+  const cudaError_t e = take ? launch(attn_tc_kernel<D, kMasked, true>, kThreads<true>)
+                             : launch(attn_tc_kernel<D, kMasked, false>, kThreads<false>);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "attn_tc launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }

@@ -16,7 +16,7 @@ from test_gpu_attn import compare, rand_qkv
 
 pytestmark = pytest.mark.gpu
 
-CAUSAL, LOCAL = 1, 2
+FULL, CAUSAL, LOCAL = 0, 1, 2
 
 
 def gpu_masked(q, k, v, seq_lens, prompt_lens, mode, block):
@@ -169,3 +169,25 @@ def test_f32_tiles_across_heads(B, L, Hq, Hkv, D, mode, block):
     sl = [min(n, L) for n in sl]
     pl = [(0, n // 3, n)[b % 3] for b, n in enumerate(sl)]
     run(B, L, Hq, Hkv, D, sl, pl, mode, block, 1.0, "f32", seed=L + block + mode)
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,D", [
+    (3, 1600, 16, 2, 128),    # units taken by the CTAs that are free (12 row tiles and more)
+    (7, 1537, 6, 2, 64),      # the same, an odd number of query heads per key/value head
+    (18, 650, 12, 4, 128), (30, 513, 8, 8, 64),   # block-causal by row tile: odd group, no group
+    (40, 129, 8, 2, 128), (73, 300, 4, 1, 64),    # in the order of the heads
+])
+@pytest.mark.parametrize("mode", [FULL, CAUSAL, LOCAL])
+def test_unit_order_bit_identical(mode, B, L, Hq, Hkv, D):
+    """Which CTA computes a unit, and when, changes nothing: each sequence of a
+    ragged batch as in a call of its own, where every unit has its own CTA."""
+    q, k, v = (t.to(dev()) for t in rand_qkv(B, L, Hq, Hkv, D, 1.0, "bf16", L + mode))
+    sl = [(L, 1, 0, L - 1, 128, L // 2, 129)[b % 7] for b in range(B)]
+    sl = [min(n, L) for n in sl]
+    pl = [(0, n // 3, n)[b % 3] for b, n in enumerate(sl)]
+    out = gpu_masked(q, k, v, sl, pl, mode, 64)
+    for b in range(0, B, max(1, B // 14)):
+        one = gpu_masked(q[b:b + 1], k[b:b + 1], v[b:b + 1], sl[b:b + 1], pl[b:b + 1], mode, 64)
+        assert torch.equal(out[b:b + 1], one), f"sequence {b}"
+    again = gpu_masked(q, k, v, sl, pl, mode, 64)
+    assert torch.equal(out, again)
