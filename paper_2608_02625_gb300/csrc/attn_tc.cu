@@ -64,6 +64,7 @@
 #include <cmath>
 #include <cstdint>
 #include <mutex>
+#include <numeric>
 
 #include "dlm_common.cuh"
 #include "dlm_internal.h"
@@ -909,11 +910,20 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   // anyway (8 x 2048 404 / 411): up to 10 rounds.
   const long long rounds = (units + sms - 1) / sms;
   const bool take = a.mask_mode != DLM_ATTN_BLOCK_LOCAL && p.mtiles >= 12 && units > sms && rounds <= 10;
+  // Block-causal units of the later row tiles have more keys: by row tile, the last
+  // first, the longest units begin first and the CTAs' shares are alike. In the
+  // order of the heads a CTA takes every gcd(grid, units per head)-th unit of a head
+  // in turn, which is as good where that skips no row tile and comes round, or
+  // skips few of many and comes round twice (73 x 865 (4 / 1) 75 us, by row tile 78;
+  // 16 x 2048 415 / 440: units of one length begin and end together on all SMs), but
+  // not else (32 x 512 112 us, by row tile 107; 18 x 650 (12 / 4) 51 / 40; 73 x 787 (8 / 8)
+  // 160 / 123; 8 x 1087 (16 / 2) 44 / 38; 34 x 130 (8 / 2) 12.2 / 9.4; 8 x 2048 260 / 247).
   const int tile_units = p.G % p.tpu == 0 ? p.G / p.tpu : 1;
+  const int step = std::gcd(sms, p.units_per_bg), turn = p.units_per_bg / step;
+  const bool even = step <= tile_units ? rounds >= turn : 4 * step <= p.units_per_bg && rounds >= 2 * turn;
   p.level_units = p.units;
   p.u_top = 0;
-  if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL && take) {
-    // By row tile, the last and so the longest units first.
+  if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL && units > sms && (take || !even)) {
     p.u_top = p.units_per_bg - tile_units;
     p.units_per_bg = tile_units;
     p.level_units = tile_units * a.B * a.Hkv;
