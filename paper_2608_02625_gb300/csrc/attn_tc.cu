@@ -143,6 +143,7 @@ struct TcParams {
   FastDiv div_upb, div_hkv, div_g;  // by units_per_bg, Hkv, G
   FastDiv div_level;  // by level_units (block masks)
   int level_units, u_top;  // units of a level, a head's first unit of level 0
+  int pairs;  // units of two tiles; those after them have one, two for a unit split
   int mask_mode, block;
   const int32_t* seq_lens;
   const int32_t* prompt_lens;
@@ -170,6 +171,8 @@ struct Unit {
 template <bool kMasked>
 __device__ __forceinline__ Unit decode_unit(const TcParams& p, int unit) {
   Unit U;
+  const int one = kMasked ? -1 : unit - p.pairs;  // >= 0: tile one % 2 of unit pairs + one / 2
+  if (one >= 0) unit = p.pairs + (one >> 1);
   // Head after head (one level), or by row tile, the last first, the units of one
   // row tile and key/value head side by side (a level per row tile).
   const int level = kMasked ? p.div_level.div(unit) : 0;
@@ -186,7 +189,7 @@ __device__ __forceinline__ Unit decode_unit(const TcParams& p, int unit) {
   U.n = n;
   const int ntiles = p.G * p.mtiles;
   {
-    const int t0 = p.tpu * u, t1 = p.tpu == 2 ? t0 + 1 : ntiles;
+    const int t0 = p.tpu * u + (one >= 0 ? one & 1 : 0), t1 = p.tpu == 2 && one < 0 ? t0 + 1 : ntiles;
     U.active.v0 = t0 < ntiles;
     U.active.v1 = t1 < ntiles;
     const int r0 = p.div_g.div(t0), r1 = p.div_g.div(t1);
@@ -899,17 +902,19 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   p.wait_ns = wait_budget_ns();
   const size_t smem = sizeof(Smem<D>) + 1024;
   // Units differ in length: by their sequence, by padding, under the block-causal
-  // mask by their row tile. Long sequences (12 row tiles): one CTA per unit is
-  // launched and whichever running CTA is free takes the next, instead of a fixed
-  // share per CTA (4 x 1836, n = 1241 .. 1633, 32 / 4 heads: 120 us against 151; 13 x 1685 (4 / 1
-  // heads) 46 / 64; 28 x 1914 (4 / 1, D = 64) 103 / 119; block-causal 2 x 2146 26 / 38, 35 x
-  // 1897 (4 / 1) 62 / 82; 5 x 2073, nearly all of one length, 168 / 166). On the whole GPU a
-  // unit is taken every 35 to 60 ns at best, which many short ones outrun (41 x
-  // 1664, n = 445 .. 455, 2132 units 76 / 71, block-causal 83 / 66; 32 x 512 block-causal
-  // 112 / 107), and where there are many rounds of them shares are nearly even
-  // anyway (8 x 2048 404 / 411): up to 10 rounds.
+  // mask by their row tile. One CTA per unit is launched and whichever running CTA is
+  // free takes the next, instead of a fixed share per CTA (4 x 1836, n = 1241 .. 1633,
+  // 32 / 4 heads 117 us against 151; 13 x 1685 (4 / 1) 45 / 64; 2 x 577 (32 / 4) 14 / 21; 14 x
+  // 1107 (8 / 2, D = 64) 24 / 29; block-causal 2 x 2146 25 / 38, 35 x 1897 (4 / 1) 61 / 82, 9 x 1158
+  // (8 / 8) 34 / 42; 5 x 2073, nearly all of one length, 167 / 165). On the whole GPU a unit
+  // is taken every 35 to 60 ns at best, which many short ones outrun (41 x 1664, n =
+  // 445 .. 455, 2132 units 76 / 71, block-causal 83 / 66; 34 x 692 (12 / 4) 61 / 58; 32 x 512
+  // block-causal 112 / 107; 29 x 600 (8 / 2) 25 / 24), and many rounds of them are shared
+  // nearly evenly anyway: up to 10 rounds from 12 row tiles on, up to 5 from 4 (8
+  // under the block-causal mask, whose units are half as long).
   const long long rounds = (units + sms - 1) / sms;
-  const bool take = a.mask_mode != DLM_ATTN_BLOCK_LOCAL && p.mtiles >= 12 && units > sms && rounds <= 10;
+  const bool take = a.mask_mode != DLM_ATTN_BLOCK_LOCAL && units > sms && p.mtiles >= (kMasked ? 8 : 4) &&
+                    rounds <= (p.mtiles >= 12 ? 10 : 5);
   // Block-causal units of the later row tiles have more keys: by row tile, the last
   // first, the longest units begin first and the CTAs' shares are alike. In the
   // order of the heads a CTA takes every gcd(grid, units per head)-th unit of a head
@@ -930,7 +935,20 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   }
   p.div_level = make_fastdiv(p.level_units);
   p.div_upb = make_fastdiv(p.units_per_bg);
-  const int grid = static_cast<int>(take || units < sms ? units : sms);
+  // Full attention, a last round of units for at most half the CTAs: those units as two
+  // of one tile each, which take ~0.8 of the time (taken one by one: 5 x 512 27.9 -> 25.5 us,
+  // 3 x 512 20.3 -> 18.2, 4 x 1725 (8 / 2 heads) 53.9 -> 45.8; shares: 20 x 128 15.0 -> 14.2, 24 x
+  // 188 (8 / 2) 10.6 -> 10.0). Not in shares of many rounds, where it gives least (32 x 512
+  // 118.8 -> 117.7) and padding can turn it (18 x 605 (32 / 4, D = 64) 39 -> 42), nor under the
+  // block masks, whose last units are short or of one tile (18 x 650 block-causal, 12 / 4
+  // 39 -> 43).
+  p.pairs = 0x7FFFFFFF;
+  if (!kMasked && p.tpu == 2 && !forced && p.G * p.mtiles % 2 == 0 && units > sms && rounds <= (take ? 10 : 6) &&
+      2 * (units % sms) <= sms) {
+    p.pairs = static_cast<int>(units - units % sms);
+    p.units += static_cast<int>(units % sms);
+  }
+  const int grid = take || p.units < sms ? p.units : sms;
   // Under the block masks the units differ in length, and a launch whose CTAs
   // take their places one by one is laid out worse: an ordinary launch there
   // (32 x 512 block-causal 111 us against 114; full attention the other way

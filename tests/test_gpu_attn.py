@@ -295,3 +295,31 @@ def test_f32_unaligned_views(L, Hq):
     out = view(torch.full(q.shape, float("nan")))
     gpu_attn(view(q), view(k), view(v), [L - 3], out=out)
     compare(out, ref, [L - 3], ATTN_TOL_F32, where=f"unaligned f32 L={L}")
+
+
+@pytest.mark.parametrize("B,L,Hq,Hkv,D", [
+    (10, 257, 16, 2, 128),   # 240 units: one round, then 88 units of two tiles each as they are
+    (25, 256, 8, 1, 64),     # 200 units: one round, then 48 of two tiles as 96 of one
+    (28, 256, 8, 1, 128),    # 224 units: the last 72, all but four CTAs of the second round
+    (9, 384, 12, 2, 128),    # 162 units: the last 10
+    (77, 129, 2, 1, 64),     # 154 units of two row blocks of a head each
+    (5, 512, 32, 4, 64),     # 320 units taken one by one, the last 16 as 32
+])
+def test_last_round_as_single_tiles(B, L, Hq, Hkv, D):
+    """On 152 SMs: a last round of units for at most half the CTAs runs as units of
+    one tile, bit-identical to the same tiles in units of two."""
+    from paper_2608_02625_gb300 import binding as Bn
+    q, k, v = (t.to(dev()) for t in rand_qkv(B, L, Hq, Hkv, D, 1.0, "bf16", B))
+    n = torch.tensor([(L, L - 1, 1, 0, 128)[b % 5] for b in range(B)], dtype=torch.int32, device=dev())
+    outs = []
+    for tiles in (0, 2):
+        out = torch.full(q.shape, float("nan"), dtype=q.dtype, device=dev())
+        Bn.dlm_set_attn_tiles_per_unit(tiles)
+        try:
+            Bn.dlm_bidir_attn(q, k, v, n, out)
+        finally:
+            Bn.dlm_set_attn_tiles_per_unit(0)
+        torch.cuda.synchronize()
+        assert Bn.device_error(clear=True) == 0
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])

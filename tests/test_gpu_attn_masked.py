@@ -174,6 +174,7 @@ def test_f32_tiles_across_heads(B, L, Hq, Hkv, D, mode, block):
 @pytest.mark.parametrize("B,L,Hq,Hkv,D", [
     (3, 1600, 16, 2, 128),    # units taken by the CTAs that are free (12 row tiles and more)
     (7, 1537, 6, 2, 64),      # the same, an odd number of query heads per key/value head
+    (6, 1100, 6, 2, 64), (4, 577, 16, 4, 128),    # the same in few rounds, full attention of 4 row tiles and more
     (18, 650, 12, 4, 128), (30, 513, 8, 8, 64),   # block-causal by row tile: odd group, no group
     (40, 129, 8, 2, 128), (73, 300, 4, 1, 64),    # in the order of the heads
 ])
