@@ -12,12 +12,12 @@
 // Integer work and exact fp32 compares only: results are bit-exact.
 //
 // Bound by latency: a few KB per sequence, one chain of loads, a selection and
-// stores. refine_update_kernel holds a sequence of up to 8 positions per
+// stores. refine_update_kernel holds a sequence of up to 16 positions per
 // thread in registers: every load of a thread is issued before any waits (by
 // position, so that not even the lengths come first), the selection takes one
 // barrier per 5 bits of the key and ends as soon as the remaining ties need no
 // order, and each output is written once. From a CUDA graph: 8 x 2048 8.7 -> 6.4
-// us, 32 x 512 5.8 -> 4.1, 4 x 64 5.6 -> 2.9, 1 x 8192 36.5 -> 15.4 against the walk in
+// us, 32 x 512 5.8 -> 4.1, 4 x 64 5.6 -> 2.9, 1 x 8192 18.0 -> 13.6 against the walk in
 // passes (refine_sequence, update_impl.cuh), which longer sequences still take.
 #include <cmath>
 #include <cstdint>
@@ -233,10 +233,13 @@ int launch(const UpdateArgs& a, cudaStream_t stream) {
   const dim3 grid(static_cast<unsigned>(a.B));
   int* err = device_error_word();
   cudaError_t e;
-  // The fewest threads that hold the sequence: fewer warps meet at each barrier.
+  // The fewest threads that hold the sequence: fewer warps meet at each barrier (35
+  // sequences of 2049 / 4096 / 8192 positions: 512 threads 6.9 / 8.8 / 16.0 us, 1024 threads with 8
+  // positions each 10.0 / 11.4 / 17.7, the walk in passes 7.8 / 10.6 / 18.4).
   if (a.L <= 512) e = launch_overlapped(refine_update_kernel<128, 4, kAfterVocab>, grid, 128, 0, stream, 1, true, a, err);
   else if (a.L <= 2048) e = launch_overlapped(refine_update_kernel<256, 8, kAfterVocab>, grid, 256, 0, stream, 1, true, a, err);
-  else if (a.L <= 8192) e = launch_overlapped(refine_update_kernel<1024, 8, kAfterVocab>, grid, 1024, 0, stream, 1, true, a, err);
+  else if (a.L <= 4096) e = launch_overlapped(refine_update_kernel<512, 8, kAfterVocab>, grid, 512, 0, stream, 1, true, a, err);
+  else if (a.L <= 8192) e = launch_overlapped(refine_update_kernel<512, 16, kAfterVocab>, grid, 512, 0, stream, 1, true, a, err);
   else e = launch_overlapped(refine_update_long_kernel, grid, kLongThreads, 0, stream, 1, true, a, err);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "refine_update launch: %s", cudaGetErrorString(e));
   return DLM_OK;

@@ -149,10 +149,11 @@ def test_key_cache_boundary(r):
 
 
 @pytest.mark.parametrize("kind", ["distinct", "ties", "one_value", "neighbours", "signs"])
-@pytest.mark.parametrize("L", [127, 128, 129, 511, 512, 513, 2047, 2048, 2049, 8191, 8192, 8193])
+@pytest.mark.parametrize("L", [127, 128, 129, 511, 512, 513, 2047, 2048, 2049, 4095, 4096, 4097, 8191,
+                               8192, 8193])
 def test_register_path_edges(L, kind):
     """The edges of the launches that hold a sequence in registers (L up to 512,
-    2048 and 8192) and the first length past them: selections that end early,
+    2048, 4096 and 8192) and the first length past them: selections that end early,
     at the last two bits of the key, and in ties taken in index order."""
     rng = np.random.default_rng(L)
     B = 4
