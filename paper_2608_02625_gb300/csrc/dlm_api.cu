@@ -142,7 +142,9 @@ int* device_error_word() {
 int active_clusters(const void* kernel, int csize, int threads, size_t smem) {
   struct Known {
     const void* kernel;
-    int dev, csize, clusters;
+    int dev, csize;
+    size_t smem;
+    int clusters;
   };
   constexpr int kMax = 256;
   static std::mutex mu;
@@ -152,7 +154,7 @@ int active_clusters(const void* kernel, int csize, int threads, size_t smem) {
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
   std::lock_guard<std::mutex> lock(mu);
   for (int i = 0; i < count; ++i)
-    if (known[i].kernel == kernel && known[i].dev == dev && known[i].csize == csize) return known[i].clusters;
+    if (known[i].kernel == kernel && known[i].dev == dev && known[i].csize == csize && known[i].smem == smem) return known[i].clusters;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(csize * sms));
@@ -169,7 +171,7 @@ int active_clusters(const void* kernel, int csize, int threads, size_t smem) {
     cudaGetLastError();
     n = 0;
   }
-  if (count < kMax) known[count++] = {kernel, dev, csize, n};
+  if (count < kMax) known[count++] = {kernel, dev, csize, smem, n};
   return n;
 }
 

@@ -29,7 +29,7 @@ cudaStream_t current_stream();
 
 // Clusters of `csize` CTAs of `kernel` (`threads` each, `smem` bytes of dynamic
 // shared memory, `csize` up to 16) that run at once on the current device, 0
-// if none can; asked of the runtime once per device, kernel and size.
+// if none can; asked of the runtime once per device, kernel and sizes.
 int active_clusters(const void* kernel, int csize, int threads, size_t smem);
 
 // Launches a kernel that may start while the one before it in the stream still

@@ -409,15 +409,35 @@ __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int3
   prob[r] = p;
 }
 
+// Dynamic shared memory with which `places` CTAs of `kernel` fit on an SM (4 at
+// most, none then). A grid of fewer CTAs than the SMs have places for is launched
+// with no more places than it needs: its CTAs otherwise fill the SMs that the
+// kernel before it leaves first, several to an SM, while others stay empty. Behind
+// attention (a loop of 4 passes, 264 rows of 151552 bf16): 122 us, 92 so; 400 rows
+// 129 / 109; 160 rows, clusters of 2, 82 / 77; 100 rows, clusters of 4, 67.6 / 65.6.
+template <typename K>
+size_t smem_for(K kernel, int64_t places, size_t fixed) {
+  const size_t most = 227 * 1024 - fixed - 2048;  // 1 KB a CTA is the system's
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess) return 0;
+  return places < 4 ? 227 * 1024 / static_cast<size_t>(places) - fixed - 2048 : 0;
+}
+
 // One wave of clusters of (at most) `csize` CTAs, each taking rows in turn.
 template <bool BF16>
-int launch_cluster(const VocabArgs& a, int csize, cudaStream_t stream) {
+int launch_cluster(const VocabArgs& a, int csize, int sms, cudaStream_t stream) {
   const auto kernel = vocab_cluster_kernel<BF16>;
+  const void* k = reinterpret_cast<const void*>(kernel);
   int active = 0;
-  while ((active = active_clusters(reinterpret_cast<const void*>(kernel), csize, kThreads, 0)) == 0 && csize > 1) csize /= 2;
+  while ((active = active_clusters(k, csize, kThreads, 0)) == 0 && csize > 1) csize /= 2;
   if (active == 0) return fail(DLM_ERR_CUDA, "vocab_confidence: no cluster launch fits the device");
   const int64_t nclusters = a.N < active ? a.N : active;
-  const cudaError_t e = launch_overlapped(kernel, dim3(static_cast<unsigned>(nclusters * csize)), kThreads, 0, stream, csize, true, a);
+  size_t smem = 0;
+  for (int64_t places = (nclusters * csize + sms - 1) / sms; places < 4; ++places) {
+    smem = smem_for(kernel, places, sizeof(Partial) * 2 * kMaxCluster * kWarps);
+    if (active_clusters(k, csize, kThreads, smem) >= nclusters) break;
+    smem = 0;
+  }
+  const cudaError_t e = launch_overlapped(kernel, dim3(static_cast<unsigned>(nclusters * csize)), kThreads, smem, stream, csize, true, a);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence cluster launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
@@ -456,9 +476,9 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
     const int csize = a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4;
     const int most = BF16 && row_bytes <= 200000 ? 3 * sms / 4
                                                  : active_clusters(reinterpret_cast<const void*>(vocab_cluster_kernel<BF16>), 4, kThreads, 0);
-    if (csize > 4 || a.N <= most) return launch_cluster<BF16>(a, csize, stream);
+    if (csize > 4 || a.N <= most) return launch_cluster<BF16>(a, csize, sms, stream);
   } else if (BF16 && row_bytes >= 100000 && a.N > sms && 3 * a.N <= 4 * sms) {
-    return launch_cluster<BF16>(a, 2, stream);
+    return launch_cluster<BF16>(a, 2, sms, stream);
   }
   cudaError_t e;
   const auto grid = [&](int64_t ctas) { return dim3(static_cast<unsigned>(ctas < 64 * resident ? ctas : 64 * resident)); };
@@ -467,7 +487,9 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
   else if (a.N > 3LL * sms && a.N <= resident)
     e = launch_overlapped(vocab_rows_kernel<BF16, false>, grid(a.N), kThreads, 0, stream, 1, true, a);
   else
-    e = launch_overlapped(vocab_rows_kernel<BF16, true>, grid(a.N), kThreads, 0, stream, 1, true, a);
+    e = launch_overlapped(vocab_rows_kernel<BF16, true>, grid(a.N), kThreads,
+                          smem_for(vocab_rows_kernel<BF16, true>, (a.N + sms - 1) / sms, sizeof(uint4) * kStages * kThreads), stream,
+                          1, true, a);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
