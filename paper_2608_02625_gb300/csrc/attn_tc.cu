@@ -949,13 +949,15 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
     p.units += static_cast<int>(units % sms);
   }
   const int grid = take || p.units < sms ? p.units : sms;
-  // Under the block masks the units differ in length, and a launch whose CTAs
-  // take their places one by one is laid out worse: an ordinary launch there
-  // (32 x 512 block-causal 111 us against 114; full attention the other way
-  // round, 5 x 512 29.6 against 31.6, 1 x 512 9.9 against 10.1).
+  // Overlapping the launch before takes 0.6 to 1 us off a call (1 x 80 (4 / 1 heads)
+  // block-causal 5.8 -> 5.1, 5 x 96 (8 / 8) 6.7 -> 5.9, 34 x 130 (8 / 2) 9.4 -> 8.7, 68 x 938 (12 / 4)
+  // block-local 190 -> 186), but lays the CTAs out worse, as they take their places one by
+  // one; under the block masks and over many rounds that costs more (32 x 512
+  // block-causal 106.2 -> 107.9, 114 x 280 (16 / 2) block-local 80.2 -> 82.9).
+  const bool overlap = !kMasked || rounds <= 12;
   const auto launch = [&](auto kernel, int threads) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    return e != cudaSuccess ? e : launch_overlapped(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, stream, 1, !kMasked,
+    return e != cudaSuccess ? e : launch_overlapped(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, stream, 1, overlap,
                                                     mq, mk, mv, mo, p);
   };
   const cudaError_t e = take ? launch(attn_tc_kernel<D, kMasked, true>, kThreads<true>)
