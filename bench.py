@@ -947,11 +947,11 @@ def run_ours(args, rank, world):
     if ranked:
         kern["update"]["kernels"] = "token_prob_kernel + refine_update_kernel (ranking by the resulting token)"
     if fused:   # the vocabulary stream and the update share one call
-        kern["vocab"]["kernel"] = "vocab_step (vocabulary reduction + update)"
+        kern["vocab"]["kernel"] = "refine_step (vocabulary reduction, then the update)"
         kern["update"] = {"ms": 0.0, "fused_into": "vocab"}
     dominant = max(("attn", "vocab"), key=lambda kk: per_kernel[kk])
     if dominant == "vocab":
-        roof = {"kernel": "vocab_step" if fused else "vocab_confidence", "bound": "hbm",
+        roof = {"kernel": "refine_step" if fused else "vocab_confidence", "bound": "hbm",
                 "achieved": kern["vocab"]["achieved_gbs"],
                 "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": kern["vocab"]["frac_of_measured_hbm"],
                 "traffic": recorded_traffic("vocab.cu", "vocab_rows_kernel",
