@@ -463,6 +463,11 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
   //   registers 19.9, clusters of 4 15.7; 256 rows 15.7 / 20.6 / 17.5; 400 rows 21.8 /
   //   23.8; 16384 rows 681 / 722) except where one wave of CTAs fills all places
   //   (512 rows: 30.5 staged, 27.7 from registers).
+  // Clusters of 16 up to 2.25 CTAs per SM (22 rows 4.9 us, 8 to a cluster 4.4; V = 300000
+  // 6.4 / 6.0; 21 rows 4.4 either way, V = 300000 5.4 / 6.0), of rows of 150 KB and less up to
+  // one CTA per SM (V = 40000, 16 rows 3.5 / 2.9; V = 64000 3.6 / 3.5), and no larger clusters
+  // than all fit at once (fp32, 35 rows 7.3 us in clusters of 16, 5.4 of 8; 75 rows 13.0 of 8,
+  // 11.8 of 4).
   // Around one row per SM (clusters of 4, of 2, a CTA per row): where the clusters of 4 no
   // longer all fit at once (152 rows 14.1 / 12.5 / 11.0, fp32 23.3 / 19.9 / 17.9) and, rows
   // of 200 KB and less in bf16, a little before (V = 100000, 100 rows 6.2 / 7.7 / 7.3, 136
@@ -473,7 +478,8 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
   // 23.6 / 20.3 / 19.2).
   if (row_bytes >= 65536 && a.N <= sms) {
     const int64_t ctas = row_bytes > 400000 ? resident : 2 * resident / 3;
-    const int csize = a.N * 16 <= ctas ? 16 : a.N * 8 <= ctas ? 8 : 4;
+    int csize = a.N * 16 <= (row_bytes > 150000 ? 9 * sms / 4 : sms) ? 16 : a.N * 8 <= ctas ? 8 : 4;
+    while (csize > 4 && a.N > active_clusters(reinterpret_cast<const void*>(vocab_cluster_kernel<BF16>), csize, kThreads, 0)) csize /= 2;
     const int most = BF16 && row_bytes <= 200000 ? 3 * sms / 4
                                                  : active_clusters(reinterpret_cast<const void*>(vocab_cluster_kernel<BF16>), 4, kThreads, 0);
     if (csize > 4 || a.N <= most) return launch_cluster<BF16>(a, csize, sms, stream);

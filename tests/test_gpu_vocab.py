@@ -211,13 +211,13 @@ def test_large_maxima_cost_no_accuracy(dtype, peak, N, V):
 
 
 @pytest.mark.parametrize("dtype,V", [("bf16", 51201), ("bf16", 110001), ("f32", 17001)])
-def test_around_one_row_per_sm(dtype, V):
-    """Clusters of 4, a CTA per row, clusters of 2 and a CTA per row again, with
-    every number of rows around which the choice turns on 152 SMs."""
+def test_choice_of_clusters(dtype, V):
+    """Clusters of 16, 8 and 4, a CTA per row, clusters of 2 and a CTA per row again,
+    with every number of rows around which the choice turns on 152 SMs."""
     x = planted(210, V, V)
     x[::7, V - 1] = 40.0
     x[::7, V // 2] = 40.0
     full = to_dev(x, dtype)
     ref = oracle.vocab_confidence(full.float().cpu().numpy())
-    for N in (113, 114, 115, 147, 148, 149, 152, 153, 202, 203, 210):
+    for N in (9, 10, 21, 22, 33, 34, 50, 51, 75, 76, 113, 114, 115, 147, 148, 149, 152, 153, 202, 203, 210):
         check_vocab(*gpu_vocab(full[:N]), *(r[:N] for r in ref), where=f"{dtype} {N}x{V}")
