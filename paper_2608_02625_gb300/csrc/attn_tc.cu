@@ -913,8 +913,12 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   // nearly evenly anyway: up to 10 rounds from 12 row tiles on, up to 5 from 4 (8
   // under the block-causal mask, whose units are half as long).
   const long long rounds = (units + sms - 1) / sms;
+  // (full attention of fewer than 12 row tiles: not two rounds of which the second is
+  // more than half full, where there is little to even out: 4 x 446, n = 149 .. 174, 12.7 us
+  // taken, 11.0 in shares; 11 x 634 (8 / 8, D = 64) 21.5 / 19.7; 4 x 512 22.0 either way).
+  const bool tail = p.tpu == 2 && !forced && p.G * p.mtiles % 2 == 0 && 2 * (units % sms) <= sms;
   const bool take = a.mask_mode != DLM_ATTN_BLOCK_LOCAL && units > sms && p.mtiles >= (kMasked ? 8 : 4) &&
-                    rounds <= (p.mtiles >= 12 ? 10 : 5);
+                    rounds <= (p.mtiles >= 12 ? 10 : 5) && (kMasked || p.mtiles >= 12 || rounds > 2 || tail);
   // Block-causal units of the later row tiles have more keys: by row tile, the last
   // first, the longest units begin first and the CTAs' shares are alike. In the
   // order of the heads a CTA takes every gcd(grid, units per head)-th unit of a head
@@ -943,8 +947,7 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   // block masks, whose last units are short or of one tile (18 x 650 block-causal, 12 / 4
   // 39 -> 43).
   p.pairs = 0x7FFFFFFF;
-  if (!kMasked && p.tpu == 2 && !forced && p.G * p.mtiles % 2 == 0 && units > sms && rounds <= (take ? 10 : 6) &&
-      2 * (units % sms) <= sms) {
+  if (!kMasked && tail && units > sms && rounds <= (take ? 10 : 6)) {
     p.pairs = static_cast<int>(units - units % sms);
     p.units += static_cast<int>(units % sms);
   }
@@ -953,8 +956,9 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   // block-causal 5.8 -> 5.1, 5 x 96 (8 / 8) 6.7 -> 5.9, 34 x 130 (8 / 2) 9.4 -> 8.7, 68 x 938 (12 / 4)
   // block-local 190 -> 186), but lays the CTAs out worse, as they take their places one by
   // one; under the block masks and over many rounds that costs more (32 x 512
-  // block-causal 106.2 -> 107.9, 114 x 280 (16 / 2) block-local 80.2 -> 82.9).
-  const bool overlap = !kMasked || rounds <= 12;
+  // block-causal 106.2 -> 107.9, 114 x 280 (16 / 2) block-local 80.2 -> 82.9, 12 rounds of 76 x
+  // 282 (16 / 2, D = 64) 48.7 -> 49.8).
+  const bool overlap = !kMasked || rounds <= 11;
   const auto launch = [&](auto kernel, int threads) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     return e != cudaSuccess ? e : launch_overlapped(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, stream, 1, overlap,
