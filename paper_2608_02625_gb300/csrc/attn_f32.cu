@@ -419,12 +419,20 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   auto tiles = [&](int m) {
     return tiles_per_head(a, a.L) ? G * ((a.L + m - 1) / m) : (G * a.L + m - 1) / m;
   };
+  // Under the block-local mask a tile of fewer rows also visits fewer key tiles: the
+  // prompt's (taken as L / 16 keys) and those its rows' blocks touch (40 x 256, 8 / 2 heads,
+  // D = 64 146 us with 128 rows, 123 with 64; 1 x 512, 32 / 4, D = 64 34 / 27; 8 x 367 with 170
+  // positions, 4 / 1, 39 with 112, 35 with 32).
+  auto key_tiles = [&](int m) {
+    if (!kMasked || a.mask_mode != DLM_ATTN_BLOCK_LOCAL) return 1.0;
+    return fmin((a.L + kKeys - 1) / kKeys, a.L / (16.0 * kKeys) + 1.0 + (m + a.block - 1.0) / kKeys);
+  };
   auto cost = [&](int m, double alone, double more) {
-    return alone + (ceil(static_cast<double>(tiles(m)) * a.B * a.Hkv / sms) - 1.0) * more;
+    return (alone + (ceil(static_cast<double>(tiles(m)) * a.B * a.Hkv / sms) - 1.0) * more) * key_tiles(m);
   };
   // 112 rows only where they make more tiles (7 x 150, 8 heads each its own: the same
   // 112 CTAs either way, 20.0 us with 128 rows and 23.8 with 112).
-  const double c8 = cost(128, 1.0, 1.0), c7 = tiles(112) > tiles(128) ? cost(112, 0.94, 0.94) : c8 + 1.0,
+  const double c8 = cost(128, 1.0, 1.0), c7 = tiles(112) > tiles(128) ? cost(112, 0.94, 0.94) : 1e300,
                c4 = cost(64, 0.7, D == 64 ? 0.54 : 0.7), c2 = cost(32, 0.55, 0.44);
   const double best = fmin(fmin(c8, c7), fmin(c4, c2));
   if (c8 == best) return launch_tile<D, 8, kMasked>(a, vec, stream);
