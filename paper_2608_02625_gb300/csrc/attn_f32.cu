@@ -252,9 +252,7 @@ __global__ void __launch_bounds__(kThreads, kR == 2 || (kR == 4 && D == 64) ? 2 
     copies_commit();
     // ---- online softmax; numerators to the half-warp's slice
     // Whether some row of the CTA may not use some key of the tile.
-    const bool partial = kMasked ? !(key0 + kKeys <= min(first.hi1, last.hi1) ||
-                                     (key0 >= last.lo2 && key0 + kKeys <= min(first.hi2, last.hi2)))
-                                 : key0 + kKeys > n;
+    const bool partial = kMasked ? !all_rows_use(first, last, key0, key0 + kKeys) : key0 + kKeys > n;
 #pragma unroll
     for (int r = 0; r < kR; ++r) {
       float s[4];

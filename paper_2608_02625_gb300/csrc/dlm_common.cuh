@@ -116,6 +116,15 @@ __host__ __device__ __forceinline__ KeyRanges key_ranges(int mode, int block, in
   return r;
 }
 
+// Whether every row from a lowest to a highest position, whose ranges are `first`
+// and `last`, may use every key of [key0, key1): the keys before the lower hi1 are
+// every row's (hi1 rises with the row), those of an own block only where both rows,
+// and so all between them, have that block (a prompt row has none: lo2 = n).
+__host__ __device__ __forceinline__ bool all_rows_use(const KeyRanges& first, const KeyRanges& last, int key0, int key1) {
+  return key1 <= (first.hi1 < last.hi1 ? first.hi1 : last.hi1) ||
+         (first.lo2 == last.lo2 && key0 >= last.lo2 && key1 <= last.hi2);
+}
+
 // Wall-clock budget of one bounded wait. Long enough for any legitimate wait
 // inside one launch, short enough that a broken pipeline ends quickly.
 constexpr uint64_t kWaitBudgetNs = 2000000000ull;  // 2 s

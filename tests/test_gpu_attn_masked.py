@@ -156,6 +156,37 @@ def test_f32_values_outside_a_mask_never_reach_a_row(mode, Hq):
     assert not torch.isfinite(got[0, attends]).any()
 
 
+@pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
+@pytest.mark.parametrize("Hq", [2, 40, 80, 152])
+def test_f32_values_of_a_block_never_reach_the_prompt(mode, Hq):
+    """The same for a key in a 64-key tile that lies wholly inside the block, of
+    which row tiles that begin in the prompt have rows as well."""
+    L, p, block, key = 200, 20, 128, 97   # blocks [20, 148), [148, 200); the tile [64, 128)
+    q, k, v = rand_qkv(1, L, Hq, 1, 64, 1.0, "f32", seed=Hq + 1)
+    bad = v.clone()
+    bad[0, key, 0, ::2] = float("nan")
+    bad[0, key, 0, 1::2] = float("inf")
+    good, got = (gpu_masked(q.to(dev()), k.to(dev()), x.to(dev()), [L], [p], mode, block) for x in (v, bad))
+    attends = torch.zeros(L, dtype=torch.bool, device=dev())
+    attends[p:p + block] = True
+    if mode == CAUSAL:
+        attends[p + block:] = True
+    assert torch.equal(got[0, ~attends], good[0, ~attends])
+    assert not torch.isfinite(got[0, attends]).any()
+
+
+@pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
+@pytest.mark.parametrize("block", [64, 100, 128, 1000])
+@pytest.mark.parametrize("B,L,Hq,Hkv,D", [
+    (2, 200, 4, 2, 64), (1, 256, 32, 4, 128), (1, 226, 40, 1, 128), (8, 256, 8, 2, 128), (1, 512, 32, 4, 128)])
+def test_f32_blocks_of_whole_key_tiles(B, L, Hq, Hkv, D, block, mode):
+    """Blocks that contain whole 64-key tiles, with row tiles of 32, 64, 112 and 128
+    rows (in this order; 128 twice) that begin in the prompt or end in a later block."""
+    for p in (10, 20, 64, 100):
+        sl, pl = [L - 5 * b for b in range(B)], [p + b for b in range(B)]
+        run(B, L, Hq, Hkv, D, sl, pl, mode, block, 1.0, "f32", seed=L + block + p + mode)
+
+
 @pytest.mark.parametrize("mode,block", [(CAUSAL, 64), (LOCAL, 64), (CAUSAL, 9), (LOCAL, 20)])
 @pytest.mark.parametrize("B,L,Hq,Hkv,D", [
     (2, 337, 24, 2, 128),    # 112-row tiles from head to head, 128-row ones per head when local
