@@ -287,7 +287,7 @@ int attn_impl(const dlm_tensor* q, const dlm_tensor* k, const dlm_tensor* v, con
   a.seq_lens = seq_lens ? static_cast<const int32_t*>(seq_lens->data) : nullptr;
   a.prompt_lens = prompt_lens && mode != DLM_ATTN_FULL ? static_cast<const int32_t*>(prompt_lens->data) : nullptr;
   a.mask_mode = mode;
-  a.block = mode != DLM_ATTN_FULL ? block : 1;
+  a.block = mode != DLM_ATTN_FULL ? dlm::mask_block(block, L) : 1;
   a.B = static_cast<int>(B);
   a.L = static_cast<int>(L);
   a.Hq = static_cast<int>(Hq);

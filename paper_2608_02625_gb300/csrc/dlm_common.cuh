@@ -92,7 +92,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Keys a query row may attend to under the attention masks of dlmrefine.h:
-// [0, hi1) and [lo2, hi2) (n_b = n, p_b = p clamped to [0, n]).
+// [0, hi1) and [lo2, hi2) (n_b = n, p_b = p clamped to [0, n]; block at most L, see mask_block).
 struct KeyRanges {
   int hi1, lo2, hi2;
 };

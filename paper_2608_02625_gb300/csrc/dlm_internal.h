@@ -53,6 +53,11 @@ cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// The block size of the block masks as the kernels take it: a sequence of up to L
+// positions fits in one block of L, and the sums of positions and blocks in
+// key_ranges then stay below 2 L whatever size the caller gives.
+inline int mask_block(int block, int64_t L) { return block < L ? block : static_cast<int>(L); }
+
 struct AttnArgs {
   const void* q;
   const void* k;

@@ -157,6 +157,13 @@ def test_f32_values_outside_a_mask_never_reach_a_row(mode, Hq):
 
 
 @pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_block_of_any_size(dtype, mode):
+    """A block of 2^31 - 1 positions: the response is one block."""
+    run(2, 300, 4, 2, 64, [300, 200], [70, 0], mode, 2 ** 31 - 1, 0.125, dtype, seed=mode)
+
+
+@pytest.mark.parametrize("mode", [CAUSAL, LOCAL])
 @pytest.mark.parametrize("Hq", [2, 40, 80, 152])
 def test_f32_values_of_a_block_never_reach_the_prompt(mode, Hq):
     """The same for a key in a 64-key tile that lies wholly inside the block, of

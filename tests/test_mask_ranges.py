@@ -1,5 +1,6 @@
-"""The attention masks' key ranges (key_ranges, all_rows_use in dlm_common.cuh),
-compiled for the host and compared with the masks' definition key by key."""
+"""The attention masks' key ranges (key_ranges and all_rows_use in dlm_common.cuh,
+mask_block in dlm_internal.h), compiled for the host and compared with the masks'
+definition key by key."""
 import os
 import shutil
 import subprocess
@@ -11,6 +12,7 @@ from paper_2608_02625_gb300 import build
 PROGRAM = r"""
 #include <cstdio>
 #include "dlm_common.cuh"
+#include "dlm_internal.h"
 
 static bool allowed(int mode, long long block, int row, int key, int p) {
   if (key < p) return true;
@@ -20,13 +22,13 @@ static bool allowed(int mode, long long block, int row, int key, int p) {
 }
 
 static int ranges() {
-  const int blocks[] = {1, 7, 64, 100, 1000};
+  const int blocks[] = {1, 7, 64, 100, 1000, 0x7FFFFFFF - 70, 0x7FFFFFFF};  // p + block overflows for the last two
   for (int mode = 1; mode <= 2; ++mode)
     for (int block : blocks)
       for (int n = 1; n <= 140; n += 3)
         for (int p = 0; p <= n; p += 9)
           for (int row = 0; row < n; ++row) {
-            const dlm::KeyRanges r = dlm::key_ranges(mode, block, row, n, p);
+            const dlm::KeyRanges r = dlm::key_ranges(mode, dlm::mask_block(block, n), row, n, p);
             for (int key = 0; key < n; ++key)
               if ((key < r.hi1 || (key >= r.lo2 && key < r.hi2)) != allowed(mode, block, row, key, p)) {
                 std::printf("mode %d block %d n %d p %d row %d key %d\n", mode, block, n, p, row, key);
@@ -38,7 +40,7 @@ static int ranges() {
 
 // A tile may count as every row's only where each row may use each of its keys.
 static int tiles() {
-  const int blocks[] = {7, 20, 64, 100, 128, 1000}, heights[] = {1, 32, 64, 112, 128}, prompts[] = {0, 10, 20, 64, 100, 128};
+  const int blocks[] = {7, 20, 64, 100, 128, 1000, 0x7FFFFFFF}, heights[] = {1, 32, 64, 112, 128}, prompts[] = {0, 10, 20, 64, 100, 128};
   int whole = 0;
   for (int mode = 1; mode <= 2; ++mode)
     for (int block : blocks)
@@ -47,7 +49,8 @@ static int tiles() {
           for (int m : heights)
             for (int r0 = 0; p <= n && r0 < n; r0 += m) {
               const int r1 = (r0 + m < n ? r0 + m : n) - 1;
-              const dlm::KeyRanges first = dlm::key_ranges(mode, block, r0, n, p), last = dlm::key_ranges(mode, block, r1, n, p);
+              const int blk = dlm::mask_block(block, n);
+              const dlm::KeyRanges first = dlm::key_ranges(mode, blk, r0, n, p), last = dlm::key_ranges(mode, blk, r1, n, p);
               for (int key0 = 0; key0 < n; key0 += 64) {
                 if (!dlm::all_rows_use(first, last, key0, key0 + 64)) continue;
                 ++whole;
