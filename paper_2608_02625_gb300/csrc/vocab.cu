@@ -131,9 +131,9 @@ __device__ __forceinline__ void fold_edge(Partial& p, float x, int e) {
 // Folds one 16-byte vector of kN values starting at element index e0: the
 // vector's maximum first (raising the running maximum rescales the sum, which
 // is rare), then the kN exponentials in pairs with packed fp32 FMA and add
-// into the two-lane running sum s2. mL is the running maximum times log2(e)
-// and stays finite (0 until the first finite maximum): an entry of -inf then
-// adds exp2(-inf) = 0 without a guard.
+// into the two-lane running sum s2. mL is the running maximum times log2(e),
+// 0 until the first finite maximum: an entry of -inf then adds exp2(-inf) = 0
+// without a guard. (Not for very large maxima: see scan_result.)
 template <int kN>
 __device__ __forceinline__ void fold_vec(Partial& p, float& mL, float2& s2, const float (&x)[kN], int e0) {
   float vm;
@@ -156,15 +156,6 @@ __device__ __forceinline__ void fold_vec(Partial& p, float& mL, float2& s2, cons
     const float2 y = ffma2(make_float2(x[j], x[j + 1]), k2, n2);
     s2 = fadd2(s2, make_float2(ex2_approx(y.x), ex2_approx(y.y)));
   }
-}
-
-// The sum of exp(x - m) from that of 2^(x log2(e) - mL): mL is m log2(e) rounded,
-// and what the rounding took (up to half an ulp of mL, the same for every term) is
-// put back: the root mean square error of conf at 1000 values a row goes from 2.1e-7
-// to 7e-8, at 300 rows of 151552 bf16 from 2.9e-7 to 2.2e-7, at the same time.
-__device__ __forceinline__ float sum_of(float m, float mL, float2 s2) {
-  const float s = s2.x + s2.y, d = fmaf(-m, kLog2e, mL);
-  return fabsf(d) < 1.f ? fmaf(s, 0.69314718f * d, s) : s;  // not for a maximum near the type's ends, or none
 }
 
 // Reduces the block's partials into warp 0's return value.
@@ -209,6 +200,38 @@ __device__ __forceinline__ float load_edge(const Row<BF16>& row, int t, bool fir
   return mine ? Vec<BF16>::load1(row.base, *e) : -INFINITY;
 }
 
+// The vectors' elements e, e + step, ... < e_end (and the kN - 1 after each) of a row,
+// each value subtracted from the maximum before it is scaled.
+template <bool BF16>
+__device__ __noinline__ Partial scan_again(const char* base, int64_t e, int64_t e_end, int step) {
+  Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
+  for (; e < e_end; e += step)
+    for (int j = 0; j < Vec<BF16>::kN; ++j) fold_edge(p, Vec<BF16>::load1(base, e + j), static_cast<int>(e) + j);
+  return p;
+}
+
+// The partial of the vectors v, v + step, ... < v_end of a row, folded into p, mL and
+// s2. The terms are 2^(x log2(e) - mL) with mL, m log2(e) rounded; what the rounding
+// took (up to half an ulp of mL, the same for every term) is put back: the root
+// mean square error of conf at 1000 values a row goes from 2.1e-7 to 7e-8, at 300 rows of
+// 151552 bf16 from 2.9e-7 to 2.2e-7, at the same time. From |m| = 2^17 on, where that is
+// more than 2^-7, or where a maximum before m was so low that the sum is not finite
+// (suppressed tokens are often set to the type's lowest value, whose product with
+// log2(e) is -inf), the vectors are read again. A look at each vector for such maxima
+// instead costs every row (256 rows of 151552 bf16 15.2 us, 16.0 to 17.6 with it).
+template <bool BF16>
+__device__ __forceinline__ Partial scan_result(const Row<BF16>& row, Partial p, float mL, float2 s2, int64_t v, int64_t v_end, int step) {
+  constexpr int kN = Vec<BF16>::kN;
+  p.s = s2.x + s2.y;
+  if (__builtin_expect(fabsf(p.m) < 131072.f && p.s < INFINITY, 1)) {
+    const float d = 0.69314718f * fmaf(-p.m, kLog2e, mL);
+    p.s = fmaf(p.s, fmaf(0.5f * d, d, d), p.s);
+  } else if (p.m != -INFINITY || p.s != 0.f) {
+    p = scan_again<BF16>(row.base, row.head + v * kN, row.head + v_end * kN, step * kN);
+  }
+  return p;
+}
+
 // Scans vectors [v_begin, v_end) of a row with kWidth threads, of which this
 // is number t, kUnroll loads in flight.
 template <bool BF16, int kWidth, int kUnroll>
@@ -245,8 +268,7 @@ __device__ __forceinline__ Partial scan_vectors(const Row<BF16>& row, int64_t v_
       }
     }
   }
-  p.s = sum_of(p.m, mL, s2);
-  return p;
+  return scan_result<BF16>(row, p, mL, s2, v_begin + t, v_end, kWidth);
 }
 
 // 16-byte asynchronous copy global -> shared (bypassing L1), and its groups.
@@ -297,8 +319,7 @@ __device__ __forceinline__ Partial scan_row_staged(const Row<BF16>& row, uint4* 
     fold_vec<kN>(p, mL, s2, x, row.head + static_cast<int>((first + static_cast<int64_t>(k) * kThreads) * kN));
   }
   cp_async_wait<0>();
-  p.s = sum_of(p.m, mL, s2);
-  return p;
+  return scan_result<BF16>(row, p, mL, s2, first, row.nvec, kThreads);
 }
 
 __device__ __forceinline__ void write_out(const VocabArgs& a, int64_t rowi, Partial p) {

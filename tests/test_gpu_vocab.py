@@ -221,3 +221,32 @@ def test_choice_of_clusters(dtype, V):
     ref = oracle.vocab_confidence(full.float().cpu().numpy())
     for N in (9, 10, 21, 22, 33, 34, 50, 51, 75, 76, 113, 114, 115, 147, 148, 149, 152, 153, 202, 203, 210):
         check_vocab(*gpu_vocab(full[:N]), *(r[:N] for r in ref), where=f"{dtype} {N}x{V}")
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N,V", [(12, 151553), (700, 1003), (300, 9001), (500, 9001)])
+def test_maxima_of_any_size(dtype, N, V):
+    """Rows whose maximum, or whose first maxima, lie anywhere between the type's
+    ends: suppressed entries at the lowest value, whole vectors of them at the
+    start of every thread, rows of nothing else; in a cluster, a warp and a CTA
+    (staged, from registers) per row."""
+    low, high = (float(f(torch.bfloat16 if dtype == "bf16" else torch.float32)) for f in
+                 (lambda t: torch.finfo(t).min, lambda t: torch.finfo(t).max))
+    rng = np.random.default_rng(V)
+    x = planted(N, V, N + V)
+    x[0, :] = low
+    x[1, :] = low
+    x[1, V - 1] = 2.5
+    x[2, :V // 2] = low
+    x[3, rng.random(V) < 0.9] = low
+    x[4, [V // 3, V // 2]] = high
+    x[5, :] = high
+    x[6, :] = np.where(rng.random(V) < 0.5, 2.5e38, 3.0e38)
+    x[7, :V - 20] = -1e30
+    x[8, :V // 2] = -3e10
+    x[9, :] = -1e9
+    x[10, :] = np.float32(2.0 ** 30) - 64.0 * rng.integers(0, 4, V).astype(np.float32)
+    x[11, :] = 300007.0 + rng.integers(-8, 1, V) / 4
+    t = to_dev(x, dtype)
+    ref = oracle.vocab_confidence(t.float().cpu().numpy())
+    check_vocab(*gpu_vocab(t), *ref, where=f"{dtype} {N}x{V}")
