@@ -72,9 +72,12 @@ __device__ __forceinline__ Partial warp_reduce(Partial p) {
   return r;
 }
 
+// 16 bytes of a stream read once. Not ld.global.nc, which is for data that nothing
+// writes while the kernel is resident: the logits' writer may still run when this
+// kernel starts (wait_for_previous).
 __device__ __forceinline__ uint4 ld_stream16(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(p));
   return v;
