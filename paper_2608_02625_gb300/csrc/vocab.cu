@@ -433,17 +433,22 @@ __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int3
   prob[r] = p;
 }
 
-// Dynamic shared memory with which `places` CTAs of `kernel` fit on an SM (4 at
-// most, none then). A grid of fewer CTAs than the SMs have places for is launched
+// Dynamic shared memory with which no more than `places` CTAs of `kernel` fit on an
+// SM (4 at most, none then). A grid of fewer CTAs than the SMs have places for is launched
 // with no more places than it needs: its CTAs otherwise fill the SMs that the
 // kernel before it leaves first, several to an SM, while others stay empty. Behind
 // attention (a loop of 4 passes, 264 rows of 151552 bf16): 122 us, 92 so; 400 rows
 // 129 / 109; 160 rows, clusters of 2, 82 / 77; 100 rows, clusters of 4, 67.6 / 65.6.
+// No more of it than that takes, and on SMs set to the most shared memory: what is
+// left of an SM's 228 KB (113 KB at one place, 76 at two, 57 at three) stays for
+// the kernels of other streams, which all of it taken keeps out until the reduction ends.
 template <typename K>
 size_t smem_for(K kernel, int64_t places, size_t fixed) {
-  const size_t most = 227 * 1024 - fixed - 2048;  // 1 KB a CTA is the system's
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)) != cudaSuccess) return 0;
-  return places < 4 ? 227 * 1024 / static_cast<size_t>(places) - fixed - 2048 : 0;
+  constexpr size_t kSm = 228 * 1024;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSm / 2 - fixed)) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+    return 0;
+  return places < 4 ? kSm / (static_cast<size_t>(places) + 1) - fixed : 0;
 }
 
 // One wave of clusters of (at most) `csize` CTAs, each taking rows in turn.

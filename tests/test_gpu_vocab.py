@@ -250,3 +250,29 @@ def test_maxima_of_any_size(dtype, N, V):
     t = to_dev(x, dtype)
     ref = oracle.vocab_confidence(t.float().cpu().numpy())
     check_vocab(*gpu_vocab(t), *ref, where=f"{dtype} {N}x{V}")
+
+
+@pytest.mark.parametrize("N", [38, 152, 304, 456])
+def test_leaves_shared_memory_to_other_streams(N):
+    """A reduction that has one to three CTAs on every SM (clusters, a CTA per row)
+    leaves a kernel of another stream that needs 50 KB of shared memory room
+    beside it: the small call, issued later, ends first."""
+    from paper_2608_02625_gb300 import binding as Bn
+    d = dev()
+    V = 2 ** 31 // N // 8 * 8               # 4.3 GB: most of a millisecond
+    x = torch.zeros(N, V, dtype=torch.bfloat16, device=d)
+    outs = [torch.empty(N, dtype=t, device=d) for t in (torch.int32, torch.float32, torch.float32)]
+    q = torch.zeros(1, 32, 1, 64, device=d)
+    k, v, out = torch.zeros_like(q), torch.zeros_like(q), torch.zeros_like(q)
+    streams = [torch.cuda.Stream(d) for _ in range(2)]
+    for _ in range(3):
+        ends = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[0]):
+            Bn.dlm_vocab_confidence(x, *outs)
+            ends[0].record()
+        with torch.cuda.stream(streams[1]):
+            Bn.dlm_bidir_attn(q, k, v, None, out)
+            ends[1].record()
+        torch.cuda.synchronize()
+    assert ends[1].elapsed_time(ends[0]) > 0.1
