@@ -140,39 +140,30 @@ int* device_error_word() {
 }
 
 int active_clusters(const void* kernel, int csize, int threads, size_t smem) {
-  struct Known {
-    const void* kernel;
-    int dev, csize;
-    size_t smem;
-    int clusters;
-  };
-  constexpr int kMax = 256;
-  static std::mutex mu;
-  static Known known[kMax];
-  static int count = 0;
-  int dev = 0, sms = 0;
+  static ClusterTable table;
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> lock(mu);
-  for (int i = 0; i < count; ++i)
-    if (known[i].kernel == kernel && known[i].dev == dev && known[i].csize == csize && known[i].smem == smem) return known[i].clusters;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(csize * sms));
-  cfg.blockDim = dim3(static_cast<unsigned>(threads));
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if ((csize > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
-      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+  return table.get({kernel, dev, csize, threads, smem}, [&] {
+    int sms = 0, n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const auto ask = [&] {
+      cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      cfg.gridDim = dim3(static_cast<unsigned>(csize * sms));
+      if (csize > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+      return cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+    };
+    if (ask() == cudaSuccess) return n;
     cudaGetLastError();
-    n = 0;
-  }
-  if (count < kMax) known[count++] = {kernel, dev, csize, smem, n};
-  return n;
+    return -1;
+  });
 }
 
 }  // namespace dlm

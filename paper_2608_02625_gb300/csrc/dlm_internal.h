@@ -2,8 +2,10 @@
 // launchers. Arguments here are already validated.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <mutex>
 
 #include "dlmrefine.h"
 
@@ -26,6 +28,41 @@ int fail(int status, const char* fmt, ...);
 void clear_error();
 // The calling thread's stream (dlm_set_stream).
 cudaStream_t current_stream();
+
+// Answers kept by everything they depend on. A query that fails (ask() < 0)
+// gives 0 for this time and is asked again the next.
+struct ClusterSizes {
+  const void* kernel;
+  int dev, csize, threads;
+  size_t smem;
+  bool operator==(const ClusterSizes& o) const {
+    return kernel == o.kernel && dev == o.dev && csize == o.csize && threads == o.threads && smem == o.smem;
+  }
+};
+
+class ClusterTable {
+ public:
+  template <typename Ask>
+  int get(const ClusterSizes& key, Ask ask) {
+    std::lock_guard<std::mutex> lock(mu_);
+    for (int i = 0; i < count_; ++i)
+      if (keys_[i] == key) return answers_[i];
+    const int n = ask();
+    if (n < 0) return 0;
+    if (count_ < kMax) {
+      keys_[count_] = key;
+      answers_[count_++] = n;
+    }
+    return n;
+  }
+
+ private:
+  static constexpr int kMax = 256;  // past these a query is asked every time
+  std::mutex mu_;
+  ClusterSizes keys_[kMax];
+  int answers_[kMax];
+  int count_ = 0;
+};
 
 // Clusters of `csize` CTAs of `kernel` (`threads` each, `smem` bytes of dynamic
 // shared memory, `csize` up to 16) that run at once on the current device, 0
