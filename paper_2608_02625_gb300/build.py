@@ -72,10 +72,23 @@ def _compile(src: str, verbose: bool, check_bounds: bool = False) -> tuple[str, 
     return obj, r.stdout + r.stderr
 
 
+def _marshal_built_for() -> str:
+    """What _marshal.so is compiled against besides its sources."""
+    import torch
+    return f"python {sys.version_info[:3]} torch {torch.__version__} cxx11 {int(torch._C._GLIBCXX_USE_CXX11_ABI)}\n"
+
+
+def _marshal_stamp() -> str:
+    return os.path.join(BUILD, "marshal.built_for")
+
+
 def _marshal_stale(force: bool) -> bool:
     src, out = os.path.join(CSRC, MARSHAL_SRC), os.path.join(PKG, MARSHAL)
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(INCLUDE, "dlmrefine.h")))
-    return force or not os.path.exists(out) or os.path.getmtime(out) < newest
+    if force or not os.path.exists(out) or os.path.getmtime(out) < newest or not os.path.exists(_marshal_stamp()):
+        return True
+    with open(_marshal_stamp()) as f:
+        return f.read() != _marshal_built_for()
 
 
 def _host_cxx(args: list[str]) -> None:
@@ -104,6 +117,8 @@ def _link_marshal(obj: str) -> None:
     _host_cxx(["-shared", obj, "-o", out + ".tmp", "-L" + PKG, "-ldlmrefine", "-Wl,-rpath,$ORIGIN", "-L" + tlib,
                "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + tlib])
     os.replace(out + ".tmp", out)
+    with open(_marshal_stamp(), "w") as f:
+        f.write(_marshal_built_for())
 
 
 def build(force: bool = False, verbose: bool = False, check_bounds: bool = False, out_dir: str | None = None) -> dict:
