@@ -87,8 +87,21 @@ def _load():
     return lib
 
 
+def _load_marshal():
+    """The native marshalling, which links against the library loaded above."""
+    path = os.path.join(_PKG, "_marshal.so")
+    hint = "build it with `python -m paper_2608_02625_gb300.build`"
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: {hint}")
+    try:
+        from . import _marshal
+    except ImportError as e:
+        raise ImportError(f"{path} does not load under this Python and torch ({e}): {hint}") from e
+    return _marshal
+
+
 lib = _load()
-from . import _marshal  # noqa: E402  (native marshalling; links against the library loaded above)
+_marshal = _load_marshal()
 
 
 def describe(t: torch.Tensor | None) -> DlmTensor | None:
