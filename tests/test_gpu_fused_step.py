@@ -1,4 +1,4 @@
-"""Steps A2 + A3 fused in one launch (dlm_refine_step) on the GPU.
+"""Steps A2 + A3 in one call (dlm_refine_step) on the GPU.
 
 Vocabulary outputs: against the oracle on host-regenerated logits (argmax
 exact, conf / lse within the tolerances of the separate call) and against the
@@ -7,7 +7,7 @@ computed from the oracle's own argmax / conf under the decision-margin protocol
 (identical wherever no conf lies within tolerance of a decision boundary), and
 bit for bit against dlm_refine_update run on the fused call's argmax / conf
 (the update is integer work and exact fp32 comparisons, so equal inputs give
-equal outputs). Each case runs twice on one workspace, which must be zero again
+equal outputs). Each case runs twice on one workspace, which must be zero
 after every call."""
 import numpy as np
 import pytest
@@ -143,7 +143,7 @@ def random_logits(rng, N, V, dtype, ties):
 @pytest.mark.parametrize("L,V,dtype", [(1, 7, "f32"), (37, 1000, "bf16"), (37, 4099, "f32"), (300, 2049, "bf16"),
                                        (129, 1, "bf16")])
 def test_random_ragged(seed, L, V, dtype):
-    """Ragged lengths (empty sequences and full ones), odd V (scalar loads), ties,
+    """Ragged lengths (empty sequences and full ones), odd V (rows off 16 bytes), ties,
     -inf entries, both remask modes, in-place update, 3-D and row-strided logits."""
     from paper_2608_02625_gb300 import binding as Bn
     rng = np.random.default_rng(97 * seed + L + V)
@@ -195,11 +195,10 @@ def test_empty_batch_needs_no_workspace():
 
 
 @pytest.mark.parametrize("r", [1023, 1024, 1025])
-def test_key_cache_boundary(r):
-    """The fused step's update at the capacity of its shared-memory key cache
-    (four keys per thread of the 256-thread vocabulary block: 1024 response
-    positions) and one past it: equal to the separate update on the same
-    predictions, and to the oracle under the decision-margin protocol."""
+def test_responses_of_about_a_thousand(r):
+    """The step's update of responses around four and five positions a thread
+    of its 256: equal to the separate update on the same predictions, and to the
+    oracle under the decision-margin protocol."""
     from paper_2608_02625_gb300 import binding as Bn
     rng = np.random.default_rng(9000 + r)
     d = dev()
@@ -227,7 +226,7 @@ def test_key_cache_boundary(r):
 
 @pytest.mark.parametrize("B,L,V", [(3, 1, 5), (2, 512, 33), (2, 513, 8), (1, 2049, 9), (1, 8193, 3)])
 def test_update_sees_the_whole_reduction(B, L, V):
-    """The update is launched while the reduction still runs: with each of its
+    """The update may start before the reduction has ended: with each of its
     launches (by L), over repeated calls on changing logits, its results are
     those of a separate update on the step's own predictions."""
     from paper_2608_02625_gb300 import binding as Bn

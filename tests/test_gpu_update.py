@@ -11,7 +11,7 @@ from paper_2608_02625_gb300 import workloads
 pytestmark = pytest.mark.gpu
 
 
-def run_gpu(tok, msk, am, cf, *, tau, k, frac, mask_id, prompt, seqlen, inplace=False):
+def run_gpu(tok, msk, am, cf, *, tau, k, frac, mask_id, prompt, seqlen, inplace=False, tok_prob=None):
     from paper_2608_02625_gb300 import binding as Bn
     d = dev()
     t_tok = torch.from_numpy(np.ascontiguousarray(tok, dtype=np.int32)).to(d)
@@ -27,7 +27,10 @@ def run_gpu(tok, msk, am, cf, *, tau, k, frac, mask_id, prompt, seqlen, inplace=
         nm = torch.full_like(t_msk, 7)
     params = Bn.RefineParams(tau, k, frac, mask_id, torch.tensor(np.asarray(prompt, dtype=np.int32), device=d),
                              torch.tensor(np.asarray(seqlen, dtype=np.int32), device=d))
-    Bn.dlm_refine_update(t_tok, t_msk, t_am, t_cf, params, nt, nm, ne)
+    if tok_prob is None:
+        Bn.dlm_refine_update(t_tok, t_msk, t_am, t_cf, params, nt, nm, ne)
+    else:
+        Bn.dlm_refine_update_ranked(t_tok, t_msk, t_am, t_cf, torch.from_numpy(tok_prob).to(d), params, nt, nm, ne)
     torch.cuda.synchronize()
     return nt.cpu().numpy(), nm.cpu().numpy(), ne.cpu().numpy()
 
@@ -128,24 +131,26 @@ def test_editable_window(lo, hi):
         assert np.array_equal(gpu[1][b, out], case["mask"][b, out])
 
 
+@pytest.mark.parametrize("ranked", [False, True])
+@pytest.mark.parametrize("L", [2090, 8230])
 @pytest.mark.parametrize("r", [2047, 2048, 2049])
-def test_key_cache_boundary(r):
-    """Responses at the capacity of the shared-memory key cache (four keys per
-    thread of the 512-thread update: 2048 positions) and one past it, heavy
-    ties included, against the oracle."""
+def test_key_cache_boundary(r, L, ranked):
+    """Response windows at the capacity of the shared-memory key cache of the walk
+    (four keys per thread of its 512: 2048 positions) and one past it, heavy ties
+    included, against the oracle: sequences too long for registers take the walk,
+    those of 2090 positions hold the same windows in registers."""
     rng = np.random.default_rng(r)
-    L = r + 40
     case = P.random_update_case(rng, B=3, L=L, V=40, ties=True)
-    case["prompt_lens"] = np.array([0, 17, 40])
+    case["prompt_lens"] = np.array([0, (L - r) // 2, L - r])
     case["seq_lens"] = case["prompt_lens"] + r
+    tp = rng.choice(np.array([0.0, 0.1, 0.25, 0.5], dtype=np.float32), (3, L)) if ranked else None
     for k, frac in ((-1, 0.1), (r // 3, 0.0), (1, 0.0)):
         ref = oracle.refine_update(case["tokens"], case["mask"], case["argmax"], case["conf"], edit_threshold=0.25,
                                    remask_k=k, remask_frac=frac, mask_id=case["V"], prompt_lens=case["prompt_lens"],
-                                   seq_lens=case["seq_lens"])
+                                   seq_lens=case["seq_lens"], tok_prob=tp)
         gpu = run_gpu(case["tokens"], case["mask"], case["argmax"], case["conf"], tau=0.25, k=k, frac=frac,
-                      mask_id=case["V"], prompt=case["prompt_lens"], seqlen=case["seq_lens"])
-        assert_same(gpu, ref, f"r={r} k={k}")
-
+                      mask_id=case["V"], prompt=case["prompt_lens"], seqlen=case["seq_lens"], tok_prob=tp)
+        assert_same(gpu, ref, f"r={r} k={k} ranked={ranked}")
 
 
 @pytest.mark.parametrize("kind", ["distinct", "ties", "one_value", "neighbours", "signs"])

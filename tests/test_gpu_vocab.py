@@ -106,7 +106,7 @@ def test_strided_rows_and_3d():
     x3 = to_dev(planted(4 * 10, V, 12), "bf16").reshape(4, 10, V)
     ref3 = oracle.vocab_confidence(x3.reshape(40, V).float().cpu().numpy())
     check_vocab(*gpu_vocab(x3), *ref3, where="3d")
-    odd = wide[:, 3:3 + V]                   # rows not 16-byte aligned: scalar path
+    odd = wide[:, 3:3 + V]                   # rows not 16-byte aligned
     ref_odd = oracle.vocab_confidence(odd.float().cpu().numpy())
     check_vocab(*gpu_vocab(odd), *ref_odd, where="unaligned")
 
