@@ -1,7 +1,7 @@
 /*
  * Test hooks exported only by DLM_CHECK_BOUNDS builds of libdlmrefine
  * (python -m paper_2608_02625_gb300.build --check-bounds --out DIR); the
- * default build does not have them. None of them is part of the method.
+ * default build does not have them. They are no part of the method.
  */
 #ifndef DLMREFINE_CHECKED_H_
 #define DLMREFINE_CHECKED_H_
@@ -11,15 +11,6 @@
 #ifdef __cplusplus
 extern "C" {
 #endif
-
-/*
- * Fills every byte of dlm_refine_step_static's static scratch on the current
- * device with `byte_value` (0..255), asynchronously on the calling thread's
- * stream, so that a test can check that no call depends on what it holds. The
- * present implementation keeps no such scratch: there is nothing to fill.
- * Returns DLM_ERR_ARG for a value outside 0..255.
- */
-int dlm_checked_fill_static_scratch(int32_t byte_value);
 
 /*
  * Sets the budget of every bounded wait in the attention and fused

@@ -671,13 +671,6 @@ int dlm_refine_step_static(const dlm_tensor* logits, const dlm_tensor* tokens, c
 #ifdef DLM_CHECK_BOUNDS
 #include "dlmrefine_checked.h"
 
-extern "C" int dlm_checked_fill_static_scratch(int32_t byte_value) {
-  using dlm::fail;
-  t_last_error[0] = '\0';
-  if (byte_value < 0 || byte_value > 255) return fail(DLM_ERR_ARG, "byte_value %d outside 0..255", byte_value);
-  return DLM_OK;
-}
-
 extern "C" int dlm_checked_set_wait_budget(int64_t budget_ns) {
   t_last_error[0] = '\0';
   if (budget_ns < 100 || budget_ns > static_cast<int64_t>(dlm::kDefaultWaitBudgetNs))

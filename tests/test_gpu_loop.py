@@ -229,8 +229,8 @@ def test_timeout_bit_stops_the_loop():
 
 
 def test_recorded_static_step_matches_oracle():
-    """The recorded pass may use dlm_refine_step_static: dlm_loop_begin sets the
-    static scratch up before the capture starts."""
+    """The recorded pass may use dlm_refine_step_static: dlm_loop_begin takes
+    the address of the device error word before the capture starts."""
     check_against_oracle(Case(2, V=8192, static=True), 8, "no_edit")
 
 

@@ -1,11 +1,11 @@
-"""dlm_refine_step_static: the fused step on the library's static scratch,
-for callers that cannot allocate device memory.
+"""dlm_refine_step_static: the step without a workspace, for callers that
+cannot allocate device memory.
 
 Collected last (conftest orders test_zz_* files after the others) and written
 to pass both alone in a fresh process, where its first call sets the device
 up, and after every other test. Each case makes two static calls in a row and
 checks both against dlm_refine_step with a caller-provided workspace, within
-the tolerances of the other vocabulary tests (the two run the same kernel, so
+the tolerances of the other vocabulary tests (the two run the same kernels, so
 the results are in fact identical)."""
 import numpy as np
 import pytest
@@ -66,8 +66,8 @@ def test_static_matches_workspace_call_twice(B, L, V):
 
 
 def test_larger_then_smaller_batch():
-    """The scratch keeps the last call's contents; a call with a smaller batch
-    after a larger one still starts from cleared counters."""
+    """A call with a smaller batch after a larger one: nothing of the first is
+    left in the second."""
     from paper_2608_02625_gb300 import binding as Bn
     for B, L, V in ((40, 64, 1000), (3, 64, 1000)):
         logits, tok, msk, params = case(B, L, V, seed=7 + B)
