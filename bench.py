@@ -441,7 +441,7 @@ def measure_fused_step(Bn, w, logits, tok, msk, params, stream, per_kernel, reps
     ms = e0.elapsed_time(e1) / reps
     sep = per_kernel["vocab"] + per_kernel["update"]
     return {"ms": ms, "ms_separate_vocab_plus_update": sep, "ratio_fused_over_separate": ms / sep,
-            "note": "dlm_refine_step (one call: the update's launch is set up while the reduction runs) on the "
+            "note": "dlm_refine_step (one call: the update starts as the reduction's last CTAs end) on the "
                     "step's buffers, against the separate calls of the step itself"}
 
 

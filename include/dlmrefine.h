@@ -266,9 +266,9 @@ int dlm_refine_update_ranked(const dlm_tensor* tokens, const dlm_tensor* mask, c
  * what dlm_vocab_confidence(logits, argmax, conf, lse) followed by
  * dlm_refine_update(tokens, mask, argmax, conf, params, new_tokens, new_mask,
  * n_edits) computes: argmax, conf and lse are written as by the first call, and
- * the update reads them back. The update's launch is set up while the
- * reduction still runs (programmatic dependent launch), so the pair costs less
- * than the two calls.
+ * the update reads them back. The update starts as the reduction's last CTAs
+ * end (programmatic dependent launch), so the pair costs less than the two
+ * calls.
  *
  *   logits  [B * L, V] or [B, L, V]   BF16 or F32, as for dlm_vocab_confidence
  *   argmax, conf, lse                 [B, L] contiguous (I32, F32, F32)

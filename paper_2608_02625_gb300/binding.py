@@ -286,7 +286,8 @@ def dlm_refine_step(logits, tokens, mask, params: RefineParams, argmax, conf, ls
     """Vocabulary reduction and refine update in one call.
 
     workspace: a CUDA tensor of at least dlm_refine_step_workspace_bytes(B) bytes,
-    zero before its first use; each completed call leaves it zero again."""
+    zero before its first use and, untouched by the present implementation, after
+    each call."""
     if _done(_marshal.refine_step(logits, tokens, mask, params, argmax, conf, lse, new_tokens, new_mask,
                                   n_edits, workspace)):
         return argmax, conf, lse, new_tokens, new_mask, n_edits

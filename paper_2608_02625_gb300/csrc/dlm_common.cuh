@@ -39,8 +39,9 @@ constexpr bool kCheckBounds = true;
 constexpr bool kCheckBounds = false;
 #endif
 
-// Every kernel of the library is launched so that it may start while the kernel
-// before it in the stream still runs (launch_overlapped, dlm_internal.h): its
+// Every kernel of a step is launched so that it may start while the kernel
+// before it in the stream still runs (launch_overlapped, dlm_internal.h; the
+// loop's own kernels and the self-test are launched the ordinary way): its
 // set-up -- barriers, tensor memory, the launch itself -- then costs nothing
 // between calls that follow each other. The rules that make this safe:
 // * no kernel touches global memory before wait_for_previous, which returns once
@@ -49,11 +50,12 @@ constexpr bool kCheckBounds = false;
 //   before it; see refine_update_kernel);
 // * no kernel lets its successor start (launch_dependents) before its own
 //   wait_for_previous, so whatever came before the predecessor has ended too.
-// Kernels of more than a few CTAs let it start when their CTAs end (which needs
-// no call), not before: CTAs that take their places one by one, as a running
-// kernel's leave, are spread unevenly over the SMs (400 vocabulary rows after
-// 400 others: 30.8 us where each CTA let the next kernel start at once, 21.7 us
-// evenly spread).
+// The reductions, fp32 attention and the projection let it start when their CTAs
+// end (which needs no call), not before: CTAs that take their places one by one,
+// as a running kernel's leave, are spread unevenly over the SMs (400 vocabulary
+// rows after 400 others: 30.8 us where each CTA let the next kernel start at once,
+// 21.7 us evenly spread). The update, short and of one CTA a sequence, does so as
+// soon as it may, bf16 attention once a CTA's last loads are issued.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Lets the next kernel of the stream take free places on the SMs once every
 // block of this one has got here or ended.

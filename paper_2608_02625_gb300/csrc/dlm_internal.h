@@ -70,7 +70,7 @@ class ClusterTable {
 int active_clusters(const void* kernel, int csize, int threads, size_t smem);
 
 // Launches a kernel that may start while the one before it in the stream still
-// runs (every kernel of the library begins with wait_for_previous), in clusters
+// runs (every kernel launched so calls wait_for_previous), in clusters
 // of `csize` CTAs; an ordinary launch where !overlap.
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int csize,
@@ -148,7 +148,7 @@ struct UpdateArgs {
 
 int launch_refine_update(const UpdateArgs& a, cudaStream_t stream);
 // The same right behind the launch_vocab_confidence that writes a.argmax and
-// a.conf, on its stream: starts before that launch has ended and waits for it.
+// a.conf, on its stream: starts when that launch's CTAs have ended and waits for its end.
 int launch_refine_update_after_vocab(const UpdateArgs& a, cudaStream_t stream);
 
 // prob[r] = exp(logits[r, tokens[r]] - lse[r]) (0 for a token outside [0, V)).

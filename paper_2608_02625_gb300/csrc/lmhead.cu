@@ -453,8 +453,8 @@ cudaError_t allow_smem() {
 }
 
 // The split that leaves the busiest CTA the fewest columns (in tiles of 256;
-// narrower tiles read the hidden rows more often: 12 % more a halving), plus a
-// small cost per item (pipeline fill, flush). Narrow tiles win where 256 columns
+// narrower tiles read the hidden rows more often: a column counts 1.12 in tiles of
+// 128 and 1.36 in tiles of 64), plus a small cost per item (pipeline fill, flush). Narrow tiles win where 256 columns
 // leave SMs without one: 16 rows x 1000 x 4096 24.3 -> 19.4 us, x 512 9.7 -> 7.5, 100 x
 // 10000 x 2048 20.6 -> 16.7, 300 x 16000 x 2048 31.6 -> 30.2. Clusters (csize > 1) run
 // one item each, all at once. Measured for 64 rows x 151552 x 2048 (reading the

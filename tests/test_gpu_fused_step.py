@@ -226,7 +226,7 @@ def test_responses_of_about_a_thousand(r):
 
 @pytest.mark.parametrize("B,L,V", [(3, 1, 5), (2, 512, 33), (2, 513, 8), (1, 2049, 9), (1, 8193, 3)])
 def test_update_sees_the_whole_reduction(B, L, V):
-    """The update may start before the reduction has ended: with each of its
+    """The update starts when the reduction's CTAs have ended, not its grid: with each of its
     launches (by L), over repeated calls on changing logits, its results are
     those of a separate update on the step's own predictions."""
     from paper_2608_02625_gb300 import binding as Bn
