@@ -479,6 +479,12 @@ int launch_step(const dlm::VocabArgs& va, const dlm::UpdateArgs& ua) {
   return st != DLM_OK ? st : dlm::launch_refine_update_after_vocab(ua, t_stream);
 }
 
+// Sequences without positions have nothing to reduce; the update counts no edits.
+int empty_step(const dlm::UpdateArgs& ua) {
+  const int st = require_error_word();
+  return st != DLM_OK ? st : dlm::launch_refine_update(ua, t_stream);
+}
+
 }  // namespace
 
 extern "C" {
@@ -627,7 +633,8 @@ int dlm_refine_step(const dlm_tensor* logits, const dlm_tensor* tokens, const dl
   dlm::UpdateArgs ua;
   int st = prepare_step(logits, tokens, mask, params, argmax, conf, lse, new_tokens, new_mask, n_edits, &va, &ua);
   if (st != DLM_OK) return st;
-  if (ua.B == 0 || va.N == 0) return DLM_OK;
+  if (ua.B == 0) return DLM_OK;
+  if (va.N == 0) return empty_step(ua);
   if (!workspace) return fail(DLM_ERR_NULL, "workspace is NULL");
   if (reinterpret_cast<uintptr_t>(workspace) % 4 != 0) return fail(DLM_ERR_ALIGN, "workspace not 4-byte aligned");
   if (workspace_bytes < dlm_refine_step_workspace_bytes(ua.B))
@@ -658,7 +665,8 @@ int dlm_refine_step_static(const dlm_tensor* logits, const dlm_tensor* tokens, c
   dlm::UpdateArgs ua;
   int st = prepare_step(logits, tokens, mask, params, argmax, conf, lse, new_tokens, new_mask, n_edits, &va, &ua);
   if (st != DLM_OK) return st;
-  if (ua.B == 0 || va.N == 0) return DLM_OK;
+  if (ua.B == 0) return DLM_OK;
+  if (va.N == 0) return empty_step(ua);
   if (ua.B > DLM_STATIC_STEP_MAX_BATCH)
     return fail(DLM_ERR_SHAPE, "batch %d exceeds the maximum of %d sequences (use dlm_refine_step)", ua.B,
                 DLM_STATIC_STEP_MAX_BATCH);

@@ -194,6 +194,25 @@ def test_empty_batch_needs_no_workspace():
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize("static", [False, True])
+def test_sequence_without_positions(static):
+    """L = 0: n_edits is written as by the separate update."""
+    from paper_2608_02625_gb300 import binding as Bn
+    d = dev()
+    z = lambda *s, dt=torch.int32: torch.empty(s, dtype=dt, device=d)
+    n = torch.zeros(1, dtype=torch.int32, device=d)
+    params = Bn.RefineParams(0.5, 1, 0.0, 9, n, n)
+    fused, separate = torch.full((1,), -1, dtype=torch.int32, device=d), torch.full((1,), -1, dtype=torch.int32, device=d)
+    tok, msk, am, cf, ls = z(1, 0), z(1, 0, dt=torch.uint8), z(1, 0), z(1, 0, dt=torch.float32), z(1, 0, dt=torch.float32)
+    Bn.dlm_refine_update(tok, msk, am, cf, params, z(1, 0), z(1, 0, dt=torch.uint8), separate)
+    args = (z(0, 16, dt=torch.bfloat16), tok, msk, params, am, cf, ls, z(1, 0), z(1, 0, dt=torch.uint8), fused)
+    if static:
+        Bn.dlm_refine_step_static(*args)
+    else:
+        Bn.dlm_refine_step(*args, z(0))
+    assert torch.equal(fused, separate) and fused.tolist() == [0]
+
+
 @pytest.mark.parametrize("r", [1023, 1024, 1025])
 def test_responses_of_about_a_thousand(r):
     """The step's update of responses around four and five positions a thread
