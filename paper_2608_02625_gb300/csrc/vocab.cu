@@ -41,6 +41,14 @@ struct Partial {
   float s;    // sum of exp(x - m)
 };
 
+// A scan starts from a maximum of -kPlain with nothing at it, so that entries far
+// below any logit (-inf, or the type's lowest value, with which tokens are often
+// suppressed) add exp2(-large) = 0 and never become the maximum that the terms are
+// relative to: times log2(e) such a maximum overflows or is rounded by more than
+// the logits' spread. A row whose maximum is not within (-kPlain, kPlain) is read
+// again (scan_any).
+constexpr float kPlain = 131072.f;  // 2^17
+
 // Order-preserving map of fp32 to int (-0 below +0).
 __device__ __forceinline__ int order_key(float x) {
   const int i = __float_as_int(x);
@@ -131,26 +139,34 @@ __device__ __forceinline__ void fold_edge(Partial& p, float x, int e) {
   }
 }
 
+// The largest of a vector's values, and the first of its elements that has it.
+template <int kN>
+__device__ __forceinline__ float vec_max(const float (&x)[kN]) {
+  if constexpr (kN == 8) return fmaxf(fmax3(fmax3(x[0], x[1], x[2]), fmax3(x[3], x[4], x[5]), x[6]), x[7]);
+  else return fmaxf(fmax3(x[0], x[1], x[2]), x[3]);
+}
+
+template <int kN>
+__device__ __forceinline__ int first_of(const float (&x)[kN], float vm) {
+  int first = kN - 1;
+#pragma unroll
+  for (int j = kN - 1; j >= 0; --j)
+    if (x[j] == vm) first = j;
+  return first;
+}
+
 // Folds one 16-byte vector of kN values starting at element index e0: the
 // vector's maximum first (raising the running maximum rescales the sum, which
 // is rare), then the kN exponentials in pairs with packed fp32 FMA and add
-// into the two-lane running sum s2. mL is the running maximum times log2(e),
-// 0 until the first finite maximum: an entry of -inf then adds exp2(-inf) = 0
-// without a guard. (Not for very large maxima: see scan_result.)
+// into the two-lane running sum s2. mL is the running maximum times log2(e).
 template <int kN>
 __device__ __forceinline__ void fold_vec(Partial& p, float& mL, float2& s2, const float (&x)[kN], int e0) {
-  float vm;
-  if constexpr (kN == 8) vm = fmaxf(fmax3(fmax3(x[0], x[1], x[2]), fmax3(x[3], x[4], x[5]), x[6]), x[7]);
-  else vm = fmaxf(fmax3(x[0], x[1], x[2]), x[3]);
+  const float vm = vec_max<kN>(x);
   if (vm > p.m) {
-    int first = kN - 1;
-#pragma unroll
-    for (int j = kN - 1; j >= 0; --j)
-      if (x[j] == vm) first = j;
-    const float up = vm * kLog2e, f = (p.m == -INFINITY) ? 0.f : ex2_approx(mL - up);
+    const float up = vm * kLog2e, f = ex2_approx(mL - up);
     s2 = make_float2(s2.x * f, s2.y * f);
     p.m = vm;
-    p.idx = e0 + first;
+    p.idx = e0 + first_of<kN>(x, vm);
     mL = up;
   }
   const float2 k2 = make_float2(kLog2e, kLog2e), n2 = make_float2(-mL, -mL);
@@ -158,6 +174,24 @@ __device__ __forceinline__ void fold_vec(Partial& p, float& mL, float2& s2, cons
   for (int j = 0; j < kN; j += 2) {
     const float2 y = ffma2(make_float2(x[j], x[j + 1]), k2, n2);
     s2 = fadd2(s2, make_float2(ex2_approx(y.x), ex2_approx(y.y)));
+  }
+}
+
+// The same for maxima of any size, from none (-inf): each value is subtracted from
+// the maximum before it is scaled.
+template <int kN>
+__device__ __forceinline__ void fold_vec_any(Partial& p, const float (&x)[kN], int e0) {
+  const float vm = vec_max<kN>(x);
+  if (vm > p.m) {
+    p.s = p.m == -INFINITY ? 0.f : p.s * ex2_approx((p.m - vm) * kLog2e);
+    p.m = vm;
+    p.idx = e0 + first_of<kN>(x, vm);
+  }
+  if (p.m != -INFINITY) {
+    float t = 0.f;  // a vector's terms first: fewer roundings of the long sum
+#pragma unroll
+    for (int j = 0; j < kN; ++j) t += ex2_approx((x[j] - p.m) * kLog2e);
+    p.s += t;
   }
 }
 
@@ -183,14 +217,15 @@ struct Row {
   const uint4* vec;  // first vector: element `head`
   int64_t nvec;
   int head, tail;
-  __device__ __forceinline__ Row(const VocabArgs& a, int64_t r) {
-    constexpr int kEsz = BF16 ? 2 : 4, kN = 16 / kEsz;
-    base = static_cast<const char*>(a.logits) + r * a.row_stride * kEsz;
+  static constexpr int kEsz = BF16 ? 2 : 4, kN = 16 / kEsz;
+  __device__ __forceinline__ Row(const VocabArgs& a, int64_t r)
+      : Row(static_cast<const char*>(a.logits) + r * a.row_stride * kEsz, a.V) {}
+  __device__ __forceinline__ Row(const char* first, int64_t V) : base(first) {
     const int64_t before = static_cast<int64_t>((0 - reinterpret_cast<uintptr_t>(base)) & 15u) / kEsz;
-    head = static_cast<int>(before < a.V ? before : a.V);
+    head = static_cast<int>(before < V ? before : V);
     vec = reinterpret_cast<const uint4*>(base + head * kEsz);
-    nvec = (a.V - head) / kN;
-    tail = static_cast<int>(a.V - head - nvec * kN);
+    nvec = (V - head) / kN;
+    tail = static_cast<int>(V - head - nvec * kN);
   }
 };
 
@@ -203,36 +238,14 @@ __device__ __forceinline__ float load_edge(const Row<BF16>& row, int t, bool fir
   return mine ? Vec<BF16>::load1(row.base, *e) : -INFINITY;
 }
 
-// The vectors' elements e, e + step, ... < e_end (and the kN - 1 after each) of a row,
-// each value subtracted from the maximum before it is scaled.
-template <bool BF16>
-__device__ __noinline__ Partial scan_again(const char* base, int64_t e, int64_t e_end, int step) {
-  Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
-  for (; e < e_end; e += step)
-    for (int j = 0; j < Vec<BF16>::kN; ++j) fold_edge(p, Vec<BF16>::load1(base, e + j), static_cast<int>(e) + j);
-  return p;
-}
-
-// The partial of the vectors v, v + step, ... < v_end of a row, folded into p, mL and
-// s2. The terms are 2^(x log2(e) - mL) with mL, m log2(e) rounded; what the rounding
-// took (up to half an ulp of mL, the same for every term) is put back: the root
-// mean square error of conf at 1000 values a row goes from 2.1e-7 to 7e-8, at 300 rows of
-// 151552 bf16 from 2.9e-7 to 2.2e-7, at the same time. From |m| = 2^17 on, where that is
-// more than 2^-7, or where a maximum before m was so low that the sum is not finite
-// (suppressed tokens are often set to the type's lowest value, whose product with
-// log2(e) is -inf), the vectors are read again. A look at each vector for such maxima
-// instead costs every row (256 rows of 151552 bf16 15.2 us, 16.0 to 17.6 with it).
-template <bool BF16>
-__device__ __forceinline__ Partial scan_result(const Row<BF16>& row, Partial p, float mL, float2 s2, int64_t v, int64_t v_end, int step) {
-  constexpr int kN = Vec<BF16>::kN;
-  p.s = s2.x + s2.y;
-  if (__builtin_expect(fabsf(p.m) < 131072.f && p.s < INFINITY, 1)) {
-    const float d = 0.69314718f * fmaf(-p.m, kLog2e, mL);
-    p.s = fmaf(p.s, fmaf(0.5f * d, d, d), p.s);
-  } else if (p.m != -INFINITY || p.s != 0.f) {
-    p = scan_again<BF16>(row.base, row.head + v * kN, row.head + v_end * kN, step * kN);
-  }
-  return p;
+// The sum of exp(x - m) from that of 2^(x log2(e) - mL): mL is m log2(e) rounded,
+// and what the rounding took (d, up to half an ulp of mL, the same for every term) is
+// put back, as e^d - 1 = d + d^2 / 2 (|d| < 2^-7 below kPlain): the root mean square
+// error of conf at 1000 values a row goes from 2.1e-7 to 7e-8, at 300 rows of 151552 bf16
+// from 2.9e-7 to 2.2e-7, at the same time.
+__device__ __forceinline__ float sum_of(float m, float mL, float2 s2) {
+  const float s = s2.x + s2.y, d = 0.69314718f * fmaf(-m, kLog2e, mL);
+  return fmaf(s, fmaf(0.5f * d, d, d), s);
 }
 
 // Scans vectors [v_begin, v_end) of a row with kWidth threads, of which this
@@ -241,8 +254,8 @@ template <bool BF16, int kWidth, int kUnroll>
 __device__ __forceinline__ Partial scan_vectors(const Row<BF16>& row, int64_t v_begin, int64_t v_end, int t) {
   using VT = Vec<BF16>;
   constexpr int kN = VT::kN;
-  Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
-  float mL = 0.f;
+  Partial p{-kPlain, 0x7FFFFFFF, 0.f};
+  float mL = -kPlain * kLog2e;
   float2 s2 = make_float2(0.f, 0.f);
   int64_t vi = v_begin + t;
   for (; vi + (kUnroll - 1) * kWidth < v_end; vi += kUnroll * kWidth) {
@@ -271,7 +284,33 @@ __device__ __forceinline__ Partial scan_vectors(const Row<BF16>& row, int64_t v_
       }
     }
   }
-  return scan_result<BF16>(row, p, mL, s2, v_begin + t, v_end, kWidth);
+  p.s = sum_of(p.m, mL, s2);
+  return p;
+}
+
+// A row whose maximum is not within (-kPlain, kPlain) again, by one warp, in every
+// lane: 0.1 ms for a row of 151552. Out of line, after everything else and in few
+// registers, as code for such rows costs all others where it is in their way: a look
+// at each vector's maximum in the scan (256 rows of 151552 bf16 15.2 us, 16.0 to 17.6
+// so), each thread's vectors read again behind its scan (1 row 3.2 / 3.4), all threads
+// of the CTA here (15 rows of 2492 1.9 / 2.0), more loads in flight here, with which five
+// CTAs of the staged scan no longer fit on an SM (740 rows of 8054 7.0 / 7.6).
+template <bool BF16>
+__device__ __noinline__ Partial scan_any(const char* base, int64_t V, int lane) {
+  const Row<BF16> row(base, V);
+  int e;
+  const float edge = load_edge(row, lane, true, true, V, &e);
+  Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
+  uint4 next = lane < row.nvec ? ld_stream16(row.vec + lane) : make_uint4(0, 0, 0, 0);
+#pragma unroll 1
+  for (int64_t v = lane; v < row.nvec; v += 32) {
+    float x[Vec<BF16>::kN];
+    Vec<BF16>::unpack(next, x);
+    if (v + 32 < row.nvec) next = ld_stream16(row.vec + v + 32);
+    fold_vec_any<Vec<BF16>::kN>(p, x, row.head + static_cast<int>(v * Vec<BF16>::kN));
+  }
+  fold_edge(p, edge, e);
+  return warp_reduce(p);
 }
 
 // 16-byte asynchronous copy global -> shared (bypassing L1), and its groups.
@@ -300,8 +339,8 @@ template <bool BF16, int kStages>
 __device__ __forceinline__ Partial scan_row_staged(const Row<BF16>& row, uint4* ring) {
   using VT = Vec<BF16>;
   constexpr int kN = VT::kN;
-  Partial p{-INFINITY, 0x7FFFFFFF, 0.f};
-  float mL = 0.f;
+  Partial p{-kPlain, 0x7FFFFFFF, 0.f};
+  float mL = -kPlain * kLog2e;
   float2 s2 = make_float2(0.f, 0.f);
   const int64_t first = threadIdx.x;
   const int nk = first < row.nvec ? static_cast<int>((row.nvec - first + kThreads - 1) / kThreads) : 0;
@@ -322,7 +361,8 @@ __device__ __forceinline__ Partial scan_row_staged(const Row<BF16>& row, uint4* 
     fold_vec<kN>(p, mL, s2, x, row.head + static_cast<int>((first + static_cast<int64_t>(k) * kThreads) * kN));
   }
   cp_async_wait<0>();
-  return scan_result<BF16>(row, p, mL, s2, first, row.nvec, kThreads);
+  p.s = sum_of(p.m, mL, s2);
+  return p;
 }
 
 __device__ __forceinline__ void write_out(const VocabArgs& a, int64_t rowi, Partial p) {
@@ -347,6 +387,7 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_rows_kernel(VocabArgs a) {
     Partial p = kStaged ? scan_row_staged<BF16, kStages>(row, ring) : scan_vectors<BF16, kThreads, 4>(row, 0, row.nvec, threadIdx.x);
     fold_edge(p, edge, e);
     p = block_reduce(p);
+    if (threadIdx.x < 32 && !(fabsf(p.m) < kPlain)) p = scan_any<BF16>(row.base, a.V, threadIdx.x);
     if (threadIdx.x == 0) write_out(a, rowi, p);
     __syncthreads();
   }
@@ -365,6 +406,7 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_short_rows_kernel(VocabArgs
     Partial p = scan_vectors<BF16, 32, 4>(row, 0, row.nvec, lane);
     fold_edge(p, edge, e);
     p = warp_reduce(p);
+    if (!(fabsf(p.m) < kPlain)) p = scan_any<BF16>(row.base, a.V, lane);
     if (lane == 0) write_out(a, rowi, p);
   }
 }
@@ -408,6 +450,7 @@ __global__ void __launch_bounds__(kThreads, 4) vocab_cluster_kernel(VocabArgs a)
       for (int j = 0; j < kMaxCluster * kWarps; j += 32)
         if (j + lane < n) q = combine(q, parts[it & 1][j + lane]);
       q = warp_reduce(q);
+      if (!(fabsf(q.m) < kPlain)) q = scan_any<BF16>(row.base, a.V, lane);
       if (lane == 0) write_out(a, rowi, q);
     }
   }
