@@ -71,23 +71,36 @@ int active_clusters(const void* kernel, int csize, int threads, size_t smem);
 
 // Launches a kernel that may start while the one before it in the stream still
 // runs (every kernel launched so calls wait_for_previous), in clusters
-// of `csize` CTAs; an ordinary launch where !overlap.
+// of `csize` CTAs; an ordinary launch where !overlap. carveout: how much of an SM's
+// shared memory and L1 is to be shared memory, in percent (-1: the driver's choice).
 template <typename... P, typename... A>
-cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int csize,
-                              bool overlap, A... args) {
+cudaError_t launch_carved(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int csize,
+                          bool overlap, int carveout, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(static_cast<unsigned>(threads));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[3];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
   cfg.attrs = attr;
-  cfg.numAttrs = csize > 1 ? 2 : 1;
+  cfg.numAttrs = 1;
+  if (csize > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs++].val.clusterDim = {static_cast<unsigned>(csize), 1, 1};
+  }
+  if (carveout >= 0) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[cfg.numAttrs++].val.sharedMemCarveout = static_cast<unsigned>(carveout);
+  }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int csize,
+                              bool overlap, A... args) {
+  return launch_carved(kernel, grid, threads, smem, stream, csize, overlap, -1, args...);
 }
 
 // The block size of the block masks as the kernels take it: a sequence of up to L

@@ -482,17 +482,20 @@ __global__ void __launch_bounds__(256) token_prob_kernel(VocabArgs a, const int3
 // kernel before it leaves first, several to an SM, while others stay empty. Behind
 // attention (a loop of 4 passes, 264 rows of 151552 bf16): 122 us, 92 so; 400 rows
 // 129 / 109; 160 rows, clusters of 2, 82 / 77; 100 rows, clusters of 4, 67.6 / 65.6.
-// No more of it than that takes, and on SMs set to the most shared memory: what is
-// left of an SM's 228 KB (113 KB at one place, 76 at two, 57 at three) stays for
-// the kernels of other streams, which all of it taken keeps out until the reduction ends.
+// No more of it than that takes, and on SMs set to the most shared memory
+// (carveout_for): what is left of an SM's 228 KB (113 KB at one place, 76 at two, 57 at
+// three) stays for the kernels of other streams, which all of it taken keeps out until
+// the reduction ends.
 template <typename K>
 size_t smem_for(K kernel, int64_t places, size_t fixed) {
   constexpr size_t kSm = 228 * 1024;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSm / 2 - fixed)) != cudaSuccess ||
-      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-    return 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSm / 2 - fixed)) != cudaSuccess) return 0;
   return places < 4 ? kSm / (static_cast<size_t>(places) + 1) - fixed : 0;
 }
+
+// Only such launches: four CTAs an SM with their loads in registers need the L1 for
+// what is in flight (56 rows of 151552 fp32 in clusters of 8 7.9 us, 8.4 without it).
+int carveout_for(size_t smem) { return smem > 0 ? cudaSharedmemCarveoutMaxShared : -1; }
 
 // One wave of clusters of (at most) `csize` CTAs, each taking rows in turn.
 template <bool BF16>
@@ -509,7 +512,7 @@ int launch_cluster(const VocabArgs& a, int csize, int sms, cudaStream_t stream) 
     if (active_clusters(k, csize, kThreads, smem) >= nclusters) break;
     smem = 0;
   }
-  const cudaError_t e = launch_overlapped(kernel, dim3(static_cast<unsigned>(nclusters * csize)), kThreads, smem, stream, csize, true, a);
+  const cudaError_t e = launch_carved(kernel, dim3(static_cast<unsigned>(nclusters * csize)), kThreads, smem, stream, csize, true, carveout_for(smem), a);
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence cluster launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
@@ -564,10 +567,10 @@ int launch_typed(const VocabArgs& a, cudaStream_t stream) {
     e = launch_overlapped(vocab_short_rows_kernel<BF16>, grid((a.N + kWarps - 1) / kWarps), kThreads, 0, stream, 1, true, a);
   else if (a.N > 3LL * sms && a.N <= resident)
     e = launch_overlapped(vocab_rows_kernel<BF16, false>, grid(a.N), kThreads, 0, stream, 1, true, a);
-  else
-    e = launch_overlapped(vocab_rows_kernel<BF16, true>, grid(a.N), kThreads,
-                          smem_for(vocab_rows_kernel<BF16, true>, (a.N + sms - 1) / sms, sizeof(uint4) * kStages * kThreads), stream,
-                          1, true, a);
+  else {
+    const size_t smem = smem_for(vocab_rows_kernel<BF16, true>, (a.N + sms - 1) / sms, sizeof(uint4) * kStages * kThreads);
+    e = launch_carved(vocab_rows_kernel<BF16, true>, grid(a.N), kThreads, smem, stream, 1, true, carveout_for(smem), a);
+  }
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, "vocab_confidence launch: %s", cudaGetErrorString(e));
   return DLM_OK;
 }
