@@ -143,6 +143,8 @@ struct TcParams {
   FastDiv div_upb, div_hkv, div_g;  // by units_per_bg, Hkv, G
   FastDiv div_level;  // by level_units (block masks)
   int level_units, u_top;  // units of a level, a head's first unit of level 0
+  int stagger;  // group g of CTAs starts its shares with round g % stagger (block masks)
+  FastDiv div_stagger, div_group;
   int pairs;  // units of two tiles; those after them have one, two for a unit split
   int mask_mode, block;
   const int32_t* seq_lens;
@@ -321,6 +323,13 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
   volatile int* abort = &sm.abort;
   wait_for_previous();
 
+  // The CTA's first unit: shares by row tile are gone round from a round that
+  // changes with the group of CTAs (launch_d).
+  int first_unit = blockIdx.x;
+  if constexpr (kMasked && !kTake) {
+    const int group = p.div_group.div(first_unit);
+    first_unit += (group - p.div_stagger.div(group) * p.stagger) * gridDim.x;
+  }
   // The unit after `unit`, -1 after the last (kTake: the one that warp 11 asked for).
   uint32_t reads = 0;
   auto next_unit = [&](int unit) -> int {
@@ -334,6 +343,10 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
       return unit;
     } else {
       unit += gridDim.x;
+      if (kMasked) {
+        if (unit >= p.units) unit = blockIdx.x;
+        return unit == first_unit ? -1 : unit;
+      }
       return unit < p.units ? unit : -1;
     }
   };
@@ -412,7 +425,7 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
       ++fills;
       return true;
     };
-    for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
+    for (int unit = first_unit; ok && unit >= 0; unit = next_unit(unit)) {
       const Unit U = decode_unit<kMasked>(p, unit);
       // Late, so that the CTAs ask in the order in which they end (2 x 2146
       // block-causal 25 us; all asking at the start of their unit 39).
@@ -517,7 +530,7 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
       int p_seen = 0;     // bar_p hand-offs consumed
       int f = 0;          // ring fills consumed
       bool ok = true;
-      for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
+      for (int unit = first_unit; ok && unit >= 0; unit = next_unit(unit)) {
         const Unit U = decode_unit<kMasked>(p, unit);
         if (U.nkv == 0) continue;
         const bool run = U.run[i];
@@ -595,7 +608,7 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
     int pvm_seen = 0;   // bar_pvm phases consumed
     int units_run = 0;  // bar_o phases consumed
     bool ok = true;
-    for (int unit = blockIdx.x; ok && unit >= 0; unit = next_unit(unit)) {
+    for (int unit = first_unit; ok && unit >= 0; unit = next_unit(unit)) {
       const Unit U = decode_unit<kMasked>(p, unit);
       const int f0 = f_next;
       if (U.nkv > 0) f_next += U.nkv + 1;
@@ -930,13 +943,24 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   const int tile_units = p.G % p.tpu == 0 ? p.G / p.tpu : 1;
   const int step = std::gcd(sms, p.units_per_bg), turn = p.units_per_bg / step;
   const bool even = step <= tile_units ? rounds >= turn : 4 * step <= p.units_per_bg && rounds >= 2 * turn;
+  // Shares by row tile are gone round from different rounds, or all CTAs would begin
+  // with the last row tiles, which in a padded batch are rows of zeros to write and
+  // nothing to compute (8 x 2048, n = 300 .. 712, 82.0 us from the same round, 72.0 so; n = 712
+  // 88.4 / 80.0; 32 x 512, n = 192 .. 256, 70.8 / 63.8; no padding: 32 x 512 106.3 / 104.9, 8 x
+  // 2048 246.9 / 247.2, 73 x 787 (8 / 8) 141.7 / 137.1, 18 x 650 (12 / 4) 50.0 / 50.5). The CTAs of
+  // one row tile and key/value head stay together, as they read the same keys and
+  // values (each from a round of its own: 32 x 512 115 us).
   p.level_units = p.units;
   p.u_top = 0;
+  p.stagger = 1;
   if (a.mask_mode == DLM_ATTN_BLOCK_CAUSAL && units > sms && (take || !even)) {
     p.u_top = p.units_per_bg - tile_units;
     p.units_per_bg = tile_units;
     p.level_units = tile_units * a.B * a.Hkv;
+    if (!take) p.stagger = static_cast<int>(units / sms);
   }
+  p.div_stagger = make_fastdiv(p.stagger);
+  p.div_group = make_fastdiv(tile_units);
   p.div_level = make_fastdiv(p.level_units);
   p.div_upb = make_fastdiv(p.units_per_bg);
   // Full attention, a last round of units for at most half the CTAs: those units as two
