@@ -143,8 +143,7 @@ struct TcParams {
   FastDiv div_upb, div_hkv, div_g;  // by units_per_bg, Hkv, G
   FastDiv div_level;  // by level_units (block masks)
   int level_units, u_top;  // units of a level, a head's first unit of level 0
-  int stagger;  // group g of CTAs starts its shares with round g % stagger (block masks)
-  FastDiv div_stagger, div_group;
+  int group, stagger;  // group g of `group` CTAs starts its shares with round g % stagger (block masks)
   int pairs;  // units of two tiles; those after them have one, two for a unit split
   int mask_mode, block;
   const int32_t* seq_lens;
@@ -325,11 +324,9 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
 
   // The CTA's first unit: shares by row tile are gone round from a round that
   // changes with the group of CTAs (launch_d).
-  int first_unit = blockIdx.x;
-  if constexpr (kMasked && !kTake) {
-    const int group = p.div_group.div(first_unit);
-    first_unit += (group - p.div_stagger.div(group) * p.stagger) * gridDim.x;
-  }
+  constexpr bool kRound = kMasked && !kTake;
+  const int own_unit = blockIdx.x;
+  const int first_unit = kRound ? own_unit + own_unit / p.group % p.stagger * static_cast<int>(gridDim.x) : own_unit;
   // The unit after `unit`, -1 after the last (kTake: the one that warp 11 asked for).
   uint32_t reads = 0;
   auto next_unit = [&](int unit) -> int {
@@ -343,8 +340,8 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
       return unit;
     } else {
       unit += gridDim.x;
-      if (kMasked) {
-        if (unit >= p.units) unit = blockIdx.x;
+      if (kRound) {
+        if (unit >= p.units) unit = own_unit;
         return unit == first_unit ? -1 : unit;
       }
       return unit < p.units ? unit : -1;
@@ -959,8 +956,7 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
     p.level_units = tile_units * a.B * a.Hkv;
     if (!take) p.stagger = static_cast<int>(units / sms);
   }
-  p.div_stagger = make_fastdiv(p.stagger);
-  p.div_group = make_fastdiv(tile_units);
+  p.group = tile_units;
   p.div_level = make_fastdiv(p.level_units);
   p.div_upb = make_fastdiv(p.units_per_bg);
   // Full attention, a last round of units for at most half the CTAs: those units as two
