@@ -326,7 +326,8 @@ __global__ void __launch_bounds__(kThreads<kTake>, 1)
   // changes with the group of CTAs (launch_d).
   constexpr bool kRound = kMasked && !kTake;
   const int own_unit = blockIdx.x;
-  const int first_unit = kRound ? own_unit + own_unit / p.group % p.stagger * static_cast<int>(gridDim.x) : own_unit;
+  int first_unit = own_unit;
+  if (kRound && p.stagger > 1) first_unit += own_unit / p.group % p.stagger * static_cast<int>(gridDim.x);
   // The unit after `unit`, -1 after the last (kTake: the one that warp 11 asked for).
   uint32_t reads = 0;
   auto next_unit = [&](int unit) -> int {
@@ -944,9 +945,11 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
   // with the last row tiles, which in a padded batch are rows of zeros to write and
   // nothing to compute (8 x 2048, n = 300 .. 712, 82.0 us from the same round, 72.0 so; n = 712
   // 88.4 / 80.0; 32 x 512, n = 192 .. 256, 70.8 / 63.8; no padding: 32 x 512 106.3 / 104.9, 8 x
-  // 2048 246.9 / 247.2, 73 x 787 (8 / 8) 141.7 / 137.1, 18 x 650 (12 / 4) 50.0 / 50.5). The CTAs of
-  // one row tile and key/value head stay together, as they read the same keys and
-  // values (each from a round of its own: 32 x 512 115 us).
+  // 2048 246.9 / 247.2, 73 x 787 (8 / 8) 141.7 / 137.1, 24 x 1100 (12 / 4) 120.1 / 117.4). The CTAs
+  // of one row tile and key/value head stay together, as they read the same keys and
+  // values (each from a round of its own: 32 x 512 115 us). Not in few rounds, where the
+  // longest units had better begin first (17 x 577 (12 / 4) 25.7 / 26.9, 18 x 650 50.2 / 51.3, 20 x
+  // 300 (8 / 8) 24.4 / 25.2).
   p.level_units = p.units;
   p.u_top = 0;
   p.stagger = 1;
@@ -954,7 +957,7 @@ int launch_d(const AttnArgs& a, cudaStream_t stream) {
     p.u_top = p.units_per_bg - tile_units;
     p.units_per_bg = tile_units;
     p.level_units = tile_units * a.B * a.Hkv;
-    if (!take) p.stagger = static_cast<int>(units / sms);
+    if (!take && rounds >= 8) p.stagger = static_cast<int>(units / sms);
   }
   p.group = tile_units;
   p.div_level = make_fastdiv(p.level_units);
